@@ -367,7 +367,9 @@ const char* mmcq_group_last_error(const mmcq_group_t* g);
  * The paper runs Mumax3's fixed kernels; here the launch shape of each pass of
  * the field evaluation is chosen per grid by timing.  The knobs change no data
  * layout and no arithmetic, so every plan computes the same field:
- *   x_rows         cells rows per block of the x passes (1 .. the rule's count);
+ *   x_rows         most cell rows per block of the x passes (1 .. the rule's
+ *                  count; a grid that so few blocks leave the GPU idle on takes
+ *                  fewer rows per block);
  *   col_groups[k]  kx tiles (y passes) or ky columns (z pass) per block of the
  *                  column passes: k = 0 the 2-D convolution, 1 the forward y,
  *                  2 the z pass, 3 the inverse y (0: not launched for this

@@ -22,7 +22,8 @@
 
 namespace mq {
 cudaError_t set_smem_limits();
-cudaError_t launch_xfwd(const Plan&, const Buffers&, const StageArgs&, int, cudaStream_t);
+cudaError_t launch_xfwd(const Plan&, const Material&, const Buffers&, const StageArgs&, int, cudaStream_t);
+int xinv_parts(const Plan&, const Buffers&, int, const SpecMap*, const Tune*);
 cudaError_t launch_xinv(const Plan&, const Material&, const Buffers&, const StageArgs&, int, cudaStream_t,
                         const SpecMap*, const Tune*);
 cudaError_t launch_convolution(const Plan&, const Buffers&, const StageArgs&, int, cudaStream_t, const Tune*);
@@ -32,6 +33,7 @@ int convolution_launches(const Plan&);
 bool col_fits(const Plan&);
 bool fft_fits(int, int);
 int rows_per_block(int, int);
+int rows_within(int, long long, int);
 int coupling_blocks(long long);
 bool x_fits(const Plan&);
 cudaError_t launch_set_m(float4*, const float*, const float*, long long, int, int, int*, cudaStream_t);
@@ -113,7 +115,9 @@ struct mmcq {
     int post_head = 0, post_count = 0;
     SpecMap spec_map{};     // TMA map of the x-half-spectrum (pipelined x inverse)
     Tune tune{{0, 0, 0, 0}, -1, -1, {-1, -1}};   // launch parameters chosen by mmcq_autotune (default: the fixed rules)
-    int rows_rule = 1;      // x-pass rows per block of the fixed rule
+    int rows_rule = 1;      // most x-pass rows per block of the fixed rule
+    int x_rows = 1;         // the same of the current plan
+    int sms = 0;            // SMs of the device
     int64_t tune_epoch = 0; // bumped when the launch parameters change (groups capture again)
 };
 
@@ -191,6 +195,14 @@ int upload_params(mmcq_t* h) {
     return MMCQ_OK;
 }
 
+// At most `most` rows per x-pass block (fewer on a grid that would otherwise
+// leave the GPU idle).
+void set_rows(mmcq_t* h, int most) {
+    h->x_rows = most;
+    h->P.R = rows_within(most, (long long)h->P.nrows * h->P.B, h->sms);
+    h->P.nblk = (h->P.nrows + h->P.R - 1) / h->P.R;
+}
+
 double ms_sum(mmcq_t* h) {
     double s = 0;
     for (float v : h->ms_host) s += v > 0 ? v : 0;
@@ -232,6 +244,9 @@ StageArgs step_args(const mmcq_t* h) {
     A.tol = (float)h->tol;
     A.record = h->record;
     A.nmodes = h->nmodes;
+    A.fin_prev = -1;
+    A.fin_here = 1;
+    A.nparts = xinv_parts(h->P, h->Bf, h->P.B, &h->spec_map, &h->tune);
     return A;
 }
 
@@ -286,7 +301,7 @@ int launch_timed(mmcq_t* h, int cls, const StageArgs& A, int nb, int part) {
         }
         CK(h, cudaEventRecord(h->events[ev], h->stream));
     }
-    if (cls == CLS_XFWD) CK(h, launch_xfwd(h->P, h->Bf, A, nb, h->stream));
+    if (cls == CLS_XFWD) CK(h, launch_xfwd(h->P, h->mat, h->Bf, A, nb, h->stream));
     else if (cls == CLS_XINV) CK(h, launch_xinv(h->P, h->mat, h->Bf, A, nb, h->stream, &h->spec_map, &h->tune));
     else CK(h, launch_conv_part(h->P, h->Bf, A, nb, h->stream, part, &h->tune));
     h->launches++;
@@ -330,9 +345,14 @@ int enqueue_steps(mmcq_t* h, int64_t n) {
     StageArgs A = step_args(h);
     const int B = h->P.B;
     for (int64_t it = 0; it < n; it++) {
+        // the scalar work of a stage is done by the next stage's x forward; a
+        // Dormand-Prince attempt's (its x forward reads the decision) and the
+        // call's last by the stage itself
         if (h->kind == KIND_RK4) {
             for (int s = 0; s < 4; s++) {
                 A.stage = s;
+                A.fin_prev = s > 0 ? s - 1 : (it > 0 ? 3 : -1);
+                A.fin_here = s == 3 && it == n - 1;
                 int r = run_stage(h, A, B);
                 if (r) return r;
             }
@@ -342,6 +362,8 @@ int enqueue_steps(mmcq_t* h, int64_t n) {
                 // after a host-side change (P-mode recomputes it every attempt)
                 if (s == 0 && h->mode == CAV_E && !h->k1_dirty) continue;
                 A.stage = s;
+                A.fin_prev = s - 1;
+                A.fin_here = s == 6;
                 int r = run_stage(h, A, B);
                 if (r) return r;
                 if (s == 0 && h->mode == CAV_E) h->k1_dirty = false;
@@ -428,9 +450,10 @@ int mmcq_create(mmcq_t** out, const mmcq_grid* g, double Ms, double Aex, double 
     P.NT = (P.hx + P.TX - 1) / P.TX;
     P.lt = 0;
     while ((1 << P.lt) < P.TX) P.lt++;
-    P.R = rows_per_block(P.L, P.nrows);
-    P.nblk = (P.nrows + P.R - 1) / P.R;
-    h->rows_rule = P.R;
+    if (cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
+        return bail(MMCQ_ERR_CUDA);
+    h->rows_rule = rows_per_block(P.L, P.nrows);
+    set_rows(h, h->rows_rule);
     if (!x_fits(P)) return bail(MMCQ_ERR_UNSUPPORTED);
     P.fd_nx = make_fastdiv((unsigned)P.nx);
     P.fd_ny = make_fastdiv((unsigned)P.ny);
@@ -451,6 +474,7 @@ int mmcq_create(mmcq_t** out, const mmcq_grid* g, double Ms, double Aex, double 
     M.alpha = (float)alpha;
     M.vc = g->dx * g->dy * g->dz;
     M.hbar = h->hbar;
+    M.inv_hbar = 1.0 / h->hbar;
 
     const long long BN = (long long)P.B * P.N;
     Buffers& Bf = h->Bf;
@@ -468,6 +492,7 @@ int mmcq_create(mmcq_t** out, const mmcq_grid* g, double Ms, double Aex, double 
     for (int k = 0; k < MAX_MODES; k++) Bf.prof[k] = nullptr;
     Bf.ip = (InstParams*)A(sizeof(InstParams) * P.B);
     Bf.st = (InstState*)A(sizeof(InstState) * P.B);
+    Bf.sc = (StageScalars*)A(sizeof(StageScalars) * P.B);
     // block partials: room for one row per block (the autotuner may lower P.R)
     Bf.xpart = (double*)A(sizeof(double) * MAX_MODES * (long long)P.B * P.nrows);
     Bf.mpart = (double*)A(sizeof(double) * 3LL * P.B * P.nrows);
@@ -1001,7 +1026,7 @@ std::string tune_key(const mmcq_t* h) {
 void tune_read(const mmcq_t* h, mmcq_tuning* t) {
     int gmax[4], zc, zr, yc, yr[2];
     conv_tunables(h->P, gmax, &zc, &zr, &yc, yr);
-    t->x_rows = h->P.R;
+    t->x_rows = h->x_rows;
     for (int k = 0; k < 4; k++) t->col_groups[k] = gmax[k] ? (h->tune.col_g[k] > 0 ? h->tune.col_g[k] : gmax[k]) : 0;
     t->z_split = zc ? (h->tune.z_split < 0 ? zr : h->tune.z_split) : -1;
     t->x_pipe = h->spec_map.valid ? (h->tune.x_pipe < 0 ? 1 : h->tune.x_pipe) : -1;
@@ -1014,7 +1039,7 @@ bool tune_apply(mmcq_t* h, const mmcq_tuning* t) {
     conv_tunables(h->P, gmax, &zc, &zr, &yc, yr);
     if (!t) {
         h->tune = Tune{{0, 0, 0, 0}, -1, -1, {-1, -1}};
-        h->P.R = h->rows_rule;
+        set_rows(h, h->rows_rule);
     } else {
         if (t->x_rows < 1 || t->x_rows > h->rows_rule) return false;
         for (int k = 0; k < 4; k++)
@@ -1028,9 +1053,8 @@ bool tune_apply(mmcq_t* h, const mmcq_tuning* t) {
         for (int k = 0; k < 2; k++) h->tune.y_split[k] = t->y_split[k];
         h->tune.z_split = t->z_split;
         h->tune.x_pipe = t->x_pipe;
-        h->P.R = t->x_rows;
+        set_rows(h, t->x_rows);
     }
-    h->P.nblk = (h->P.nrows + h->P.R - 1) / h->P.R;
     h->tune_epoch++;
     return true;
 }
@@ -1104,8 +1128,9 @@ int mmcq_autotune(mmcq_t* h, int reps, mmcq_tuning* out) {
     auto eval = [&](bool timed) -> cudaError_t {
         cudaError_t e;
         int q = 0;
+        A.nparts = xinv_parts(h->P, h->Bf, B, &h->spec_map, &h->tune);
         if (timed && (e = cudaEventRecord(ev[q++], h->stream)) != cudaSuccess) return e;
-        if ((e = launch_xfwd(h->P, h->Bf, A, B, h->stream)) != cudaSuccess) return e;
+        if ((e = launch_xfwd(h->P, h->mat, h->Bf, A, B, h->stream)) != cudaSuccess) return e;
         if (timed && (e = cudaEventRecord(ev[q++], h->stream)) != cudaSuccess) return e;
         for (int part = parts0; part <= parts1; part++) {
             if ((e = launch_conv_part(h->P, h->Bf, A, B, h->stream, part, &h->tune)) != cudaSuccess) return e;
@@ -1220,7 +1245,7 @@ int adj_field(mmcq_t* h, const Buffers& Bq, int terms) {
     A.kind = KIND_RK4; A.mode = CAV_E; A.stage = 0; A.field_only = 1; A.terms = terms; A.inst0 = 0;
     A.record = 0; A.nmodes = 1;
     const int B = h->P.B;
-    CK(h, launch_xfwd(h->P, Bq, A, B, h->stream));
+    CK(h, launch_xfwd(h->P, h->mat, Bq, A, B, h->stream));
     CK(h, launch_convolution(h->P, Bq, A, B, h->stream, &h->tune));
     CK(h, launch_xinv(h->P, h->mat, Bq, A, B, h->stream, &h->spec_map, &h->tune));
     return MMCQ_OK;
@@ -1728,6 +1753,7 @@ int mmcq_group_step(mmcq_group_t* g, int64_t n, double dt) {
         if (h->kind == KIND_DP45 && h->mode == CAV_E && h->k1_dirty) {
             StageArgs A = step_args(h);
             A.stage = 0;
+            A.fin_here = 0;     // the attempt's next x forward
             int r = run_stage(h, A, h->P.B);
             if (r) return gfail(g, r, "first stage launch failed");
             h->k1_dirty = false;

@@ -52,9 +52,9 @@ __device__ __forceinline__ void demag_product(const Plan& P, const float* __rest
     float2 k0 = __ldg(K), k1 = __ldg(K + 1), k2 = __ldg(K + 2);
     float xx = k0.x, yy = k0.y, zz = k1.x;
     float xy = sy * k1.y, xz = sz * k2.x, yz = sy * sz * k2.y;
-    float2 hx = make_float2(xx * mx.x + xy * my.x + xz * mz.x, xx * mx.y + xy * my.y + xz * mz.y);
-    float2 hy = make_float2(xy * mx.x + yy * my.x + yz * mz.x, xy * mx.y + yy * my.y + yz * mz.y);
-    float2 hz = make_float2(xz * mx.x + yz * my.x + zz * mz.x, xz * mx.y + yz * my.y + zz * mz.y);
+    float2 hx = make_float2(dot3(xx, mx.x, xy, my.x, xz, mz.x), dot3(xx, mx.y, xy, my.y, xz, mz.y));
+    float2 hy = make_float2(dot3(yy, my.x, xy, mx.x, yz, mz.x), dot3(yy, my.y, xy, mx.y, yz, mz.y));
+    float2 hz = make_float2(dot3(xz, mx.x, yz, my.x, zz, mz.x), dot3(xz, mx.y, yz, my.y, zz, mz.y));
     mx = hx; my = hy; mz = hz;
 }
 
@@ -208,13 +208,13 @@ __global__ void __launch_bounds__(256) k_zconv(Plan Pl, Buffers Bf, StageArgs A,
             const float2* mm = mcol + kz * W;
             const float2 mx = mm[0], my = mm[TX], mz = mm[2 * TX];
             const float c0 = a0 * fp[0], c1 = a1 * fp[1], c2 = a2 * fp[2];
-            v[kz] = make_float2(c0 * mx.x + c1 * my.x + c2 * mz.x, c0 * mx.y + c1 * my.y + c2 * mz.y);
+            v[kz] = make_float2(dot3(c0, mx.x, c1, my.x, c2, mz.x), dot3(c0, mx.y, c1, my.y, c2, mz.y));
         }
         if (kz > 0 && kz < P / 2) {
             const float2* mm = mcol + (P - kz) * W;
             const float2 mx = mm[0], my = mm[TX], mz = mm[2 * TX];
             const float c0 = a0 * fn[0], c1 = a1 * fn[1], c2 = a2 * fn[2];
-            v[P - kz] = make_float2(c0 * mx.x + c1 * my.x + c2 * mz.x, c0 * mx.y + c1 * my.y + c2 * mz.y);
+            v[P - kz] = make_float2(dot3(c0, mx.x, c1, my.x, c2, mz.x), dot3(c0, mx.y, c1, my.y, c2, mz.y));
         }
     }
     fft_reg<P, true>(v);
@@ -246,7 +246,7 @@ __device__ __forceinline__ void zsplit_forward(const ColArgs& C, float2* sm, int
         for (int r = 1; r < H; r++) {
             const int e = r * (32 / P);           // W_P^r = W_32^e
             if (e == 8) v[r] = make_float2(v[r].y, -v[r].x);
-            else v[r] = cmul(v[r], c_tw32[e]);
+            else v[r] = cmul(c_tw32[e], v[r]);
         }
     }
     fft_reg<H, false>(v);
@@ -273,7 +273,7 @@ __device__ __forceinline__ void zinv_transform(const float2* sm, int W, int col,
         for (int n = 1; n < H; n++) {
             const int e = n * (32 / P);           // W_P^{-n} = conj(W_32^e)
             if (e == 8) v[n] = make_float2(-v[n].y, v[n].x);
-            else { float2 w = c_tw32[e]; w.y = -w.y; v[n] = cmul(v[n], w); }
+            else v[n] = cmulc(v[n], c_tw32[e]);
         }
     }
 }
@@ -362,11 +362,14 @@ __global__ void __launch_bounds__(192, 6) k_zconv2(Plan Pl, Buffers Bf, StageArg
     const float* Kb = Bf.kern + ((long long)kyr * Pl.NT * TX + (live ? kx : 0)) * 6;
     float2* pm0 = sm + gg * 3 * TX + xx;
     const int kz0 = threadIdx.x >> lgt;           // 0 .. 5
-    auto apply = [&](float2* pm, float Kxx, float Kyy, float Kzz, float Kxy, float Kxz, float Kyz) {
+    // MIR (a constant at each use): the mirrored point, whose last row adds
+    // its terms in the other order
+    auto apply = [&](float2* pm, float Kxx, float Kyy, float Kzz, float Kxy, float Kxz, float Kyz, bool MIR) {
         const float2 mx = pm[0], my = pm[TX], mz = pm[2 * TX];
-        pm[0] = make_float2(Kxx * mx.x + Kxy * my.x + Kxz * mz.x, Kxx * mx.y + Kxy * my.y + Kxz * mz.y);
-        pm[TX] = make_float2(Kxy * mx.x + Kyy * my.x + Kyz * mz.x, Kxy * mx.y + Kyy * my.y + Kyz * mz.y);
-        pm[2 * TX] = make_float2(Kxz * mx.x + Kyz * my.x + Kzz * mz.x, Kxz * mx.y + Kyz * my.y + Kzz * mz.y);
+        pm[0] = make_float2(dot3(Kxx, mx.x, Kxy, my.x, Kxz, mz.x), dot3(Kxx, mx.y, Kxy, my.y, Kxz, mz.y));
+        pm[TX] = make_float2(dot3(Kxy, mx.x, Kyy, my.x, Kyz, mz.x), dot3(Kxy, mx.y, Kyy, my.y, Kyz, mz.y));
+        pm[2 * TX] = MIR ? make_float2(dot3(Kyz, my.x, Kxz, mx.x, Kzz, mz.x), dot3(Kyz, my.y, Kxz, mx.y, Kzz, mz.y))
+                         : make_float2(dot3(Kxz, mx.x, Kyz, my.x, Kzz, mz.x), dot3(Kxz, mx.y, Kyz, my.y, Kzz, mz.y));
     };
 #pragma unroll
     for (int it = 0; it < (P / 2 + 6) / 6; it++) {
@@ -376,8 +379,8 @@ __global__ void __launch_bounds__(192, 6) k_zconv2(Plan Pl, Buffers Bf, StageArg
             const float2* Kp = reinterpret_cast<const float2*>(Kb + kzr * zs);
             const float2 k0 = __ldg(Kp), k1 = __ldg(Kp + 1), k2 = __ldg(Kp + 2);
             const float Kxy = sy * k1.y, Kyz = sy * k2.y;
-            apply(pm0 + kzr * W, k0.x, k0.y, k1.x, Kxy, k2.x, Kyz);
-            if (kzr > 0 && kzr < P / 2) apply(pm0 + (P - kzr) * W, k0.x, k0.y, k1.x, Kxy, -k2.x, -Kyz);
+            apply(pm0 + kzr * W, k0.x, k0.y, k1.x, Kxy, k2.x, Kyz, false);
+            if (kzr > 0 && kzr < P / 2) apply(pm0 + (P - kzr) * W, k0.x, k0.y, k1.x, Kxy, -k2.x, -Kyz, true);
         } else {
             const float2 z0 = make_float2(0.f, 0.f);
             float2* pm = pm0 + kzr * W;
@@ -487,7 +490,7 @@ __global__ void __launch_bounds__(512, (FIXED && PH == 1024) ? 2 : 1) k_col_spli
             fft(v, true);
             if (J == 1) {
 #pragma unroll
-                for (int i = 0; i < NPT; i++) v[i] = cmul(v[i], conjf2(stw[out_row(i)]));
+                for (int i = 0; i < NPT; i++) v[i] = cmulc(v[i], stw[out_row(i)]);
             }
             // element i is row a + 16 (4 q + i / 4) + (PH / 4) (i % 4): below
             // PH / 2 exactly when i % 4 < 2.  The 8 elements a block gives
@@ -527,7 +530,7 @@ __global__ void __launch_bounds__(512, (FIXED && PH == 1024) ? 2 : 1) k_col_spli
             for (int n2 = 0; n2 < NPT; n2++) {
                 const int r = j + N1 * n2;
                 float2 x = (valid && r < C.n_in) ? in[r * in_r] : make_float2(0.f, 0.f);
-                if (J == 1) x = F3 ? cmul(x, n2 == 0 ? wj : cmul(wj, c_tw32[n2])) : cmul(x, stw[r]);
+                if (J == 1) x = F3 ? cmul(x, n2 == 0 ? wj : cmul(c_tw32[n2], wj)) : cmul(x, stw[r]);
                 v[n2] = x;
             }
             fft(v, false);
@@ -558,7 +561,7 @@ __global__ void __launch_bounds__(512, (FIXED && PH == 1024) ? 2 : 1) k_col_spli
 #pragma unroll
                     for (int i = 0; i < NPT; i++) {
                         const int k = out_row(i);
-                        const float2 y = cmul(v[i], conjf2(stw[k]));
+                        const float2 y = cmulc(v[i], stw[k]);
                         if (k < C.n_out) red_add_f2(out + k * out_r, y);
                     }
                 }

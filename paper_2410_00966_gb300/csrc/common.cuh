@@ -73,7 +73,7 @@ struct Material {
     float pre;        // -gamma / (1 + alpha^2)
     float alpha;
     double vc;        // cell volume
-    double hbar;
+    double hbar, inv_hbar;
 };
 
 // Per-instance parameters (set from the host).
@@ -115,6 +115,13 @@ struct Tune {
     int y_split[2]; // fixed split y passes (forward, inverse): 1 a half per block, 0 both halves; -1 = rule
 };
 
+// Scalars of the stage being evaluated, the same for every cell of an instance:
+// written by the scalar block of the x forward, read by the x inverse.
+struct StageScalars {
+    float gamma[MAX_MODES];   // Gamma_k of the stage (Eq. gammafinal / gammadiscretefinal)
+    float drive;              // factor of the Appendix C excitation
+};
+
 // Device buffers of one handle.
 struct Buffers {
     float4* m[2];     // [B][N] (x, y, z, Ms); m[mcur] is the accepted state
@@ -127,6 +134,7 @@ struct Buffers {
     float4* prof[MAX_MODES];  // [N] coupling-profile shape of each mode (or null: uniform +y)
     InstParams* ip;
     InstState* st;
+    StageScalars* sc; // [B]
     double* xpart;    // [MAX_MODES][B][x-pass blocks] FP64 partial coupling sums
     float* epart;     // [B][nrows] partial error maxima
     unsigned* counter;  // [B] blocks finished in the current kernel
@@ -152,6 +160,9 @@ struct StageArgs {
     float tol;
     int record;    // record <m> every `record` accepted steps (0: off)
     int nmodes;    // cavity modes in use (highest enabled mode + 1)
+    int fin_prev;  // x forward: finish this stage (index) of the launch before it first; -1: none
+    int fin_here;  // x inverse: its last block finishes this stage
+    int nparts;    // block partials per instance of the x inverse
 };
 
 }  // namespace mq

@@ -12,8 +12,21 @@
 
 namespace mq {
 
+// a b and a conj(b), with the one rounding of each fused product written out:
+// left to the compiler, which of the two products is fused depends on the code
+// around, and the same transform in two kernels (or in two builds) would round
+// differently.  So every plan of a grid gives the same field bit for bit, and
+// a Dormand-Prince run, whose step lengths amplify the last bits of its error
+// estimate, takes the same steps.
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
+    return make_float2(__fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, -__fmul_rn(a.x, b.y)));
+}
+// a x + b y + c z in the order of the demag product: b y rounded first.
+__device__ __forceinline__ float dot3(float a, float x, float b, float y, float c, float z) {
+    return __fmaf_rn(c, z, __fmaf_rn(a, x, __fmul_rn(b, y)));
 }
 // Complex add and subtract as paired FP32 instructions (sm_100 and later issue
 // the two component adds of a float2 as one instruction, each rounded like the
@@ -22,10 +35,10 @@ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
 
-// exp(-+ 2 pi i k / twn) from the table; inverse transforms use the conjugate.
-__device__ __forceinline__ float2 twiddle(const float2* __restrict__ tw, int k, bool inv) {
-    float2 w = __ldg(tw + k);
-    return inv ? make_float2(w.x, -w.y) : w;
+// v exp(-+ 2 pi i k / twn) from the table; inverse transforms use the conjugate.
+__device__ __forceinline__ float2 twiddled(float2 v, const float2* __restrict__ tw, int k, bool inv) {
+    const float2 w = __ldg(tw + k);
+    return inv ? cmulc(v, w) : cmul(v, w);
 }
 
 __device__ __forceinline__ void radix4(float2* v, bool inv) {
@@ -75,11 +88,11 @@ __device__ void block_fft(float2* s, int L, int nlines, int es, int ls, bool inv
                     if (R == 4) {
                         v[q][0] = p[j * es];
 #pragma unroll
-                        for (int r = 1; r < 4; r++) v[q][r] = cmul(p[(j + r * tpl) * es], twiddle(tw, r * ts, inv));
+                        for (int r = 1; r < 4; r++) v[q][r] = twiddled(p[(j + r * tpl) * es], tw, r * ts, inv);
                         radix4(v[q], inv);
                     } else {
                         float2 a = p[j * es];
-                        float2 b = cmul(p[(j + tpl) * es], twiddle(tw, ts, inv));
+                        float2 b = twiddled(p[(j + tpl) * es], tw, ts, inv);
                         v[q][2 * h] = cadd(a, b);
                         v[q][2 * h + 1] = csub(a, b);
                     }

@@ -68,9 +68,7 @@ __device__ __forceinline__ void fft_reg(float2* v) {
                 } else if (e == 8) {            // -i (forward) / +i (inverse)
                     v[s0 + k + len / 2] = INV ? make_float2(-d.y, d.x) : make_float2(d.y, -d.x);
                 } else {
-                    float2 w = c_tw32[e];
-                    if (INV) w.y = -w.y;
-                    v[s0 + k + len / 2] = cmul(d, w);
+                    v[s0 + k + len / 2] = INV ? cmulc(d, c_tw32[e]) : cmul(c_tw32[e], d);
                 }
             }
         }
@@ -107,10 +105,11 @@ __device__ __forceinline__ int col_out_row(int j, int i) {
 // when N1 > 1; every thread of the block must call this (it synchronises).
 // Twiddles come from `tw`, a table of exp(-2 pi i k / twn) for k < twn (a
 // multiple of P), in global memory (TW_SHARED = false, read through the
-// read-only cache) or in shared memory.
+// read-only cache) or in shared memory.  act: whether this thread holds a line
+// (the others only pass the barriers).
 template <int P, bool INV, bool TW_SHARED = false>
 __device__ __forceinline__ void col_fft(float2* v, float2* buf, int ld, int col, int j, const float2* __restrict__ tw,
-                                        int twn) {
+                                        int twn, bool act = true) {
     constexpr int NPT = ColShape<P>::NPT, N1 = ColShape<P>::N1, Q = ColShape<P>::Q;
     fft_reg<NPT, INV>(v);
     if (N1 == 1) return;
@@ -118,24 +117,23 @@ __device__ __forceinline__ void col_fft(float2* v, float2* buf, int ld, int col,
     const int step = twn / P;
 #pragma unroll
     for (int k2 = 1; k2 < NPT; k2++) {
-        float2 w;
-        if (TW_SHARED) {
-            w = tw[j * k2 * step];
-            if (INV) w.y = -w.y;
-        } else {
-            w = twiddle(tw, j * k2 * step, INV);
-        }
-        v[k2] = cmul(v[k2], w);
+        if (!act) break;
+        const float2 w = TW_SHARED ? tw[j * k2 * step] : __ldg(tw + j * k2 * step);
+        v[k2] = INV ? cmulc(v[k2], w) : cmul(v[k2], w);
     }
     __syncthreads();
+    if (act) {
 #pragma unroll
-    for (int k2 = 0; k2 < NPT; k2++) buf[(k2 * N1 + j) * ld + col] = v[k2];
+        for (int k2 = 0; k2 < NPT; k2++) buf[(k2 * N1 + j) * ld + col] = v[k2];
+    }
     __syncthreads();
+    if (act) {
 #pragma unroll
-    for (int q = 0; q < Q; q++) {
-        const int k2 = j * Q + q;
+        for (int q = 0; q < Q; q++) {
+            const int k2 = j * Q + q;
 #pragma unroll
-        for (int n1 = 0; n1 < N1; n1++) v[q * N1 + n1] = buf[(k2 * N1 + n1) * ld + col];
+            for (int n1 = 0; n1 < N1; n1++) v[q * N1 + n1] = buf[(k2 * N1 + n1) * ld + col];
+        }
     }
 #pragma unroll
     for (int q = 0; q < Q; q++) fft_reg<N1, INV>(v + q * N1);
@@ -188,18 +186,19 @@ __device__ __forceinline__ int col3_swz(int r) { return r + PADS * (r / N1); }
 // every factor carries at most one rounding beyond the table's.
 template <bool INV, bool TW_SHARED>
 __device__ __forceinline__ void twiddle15(float2* v, const float2* __restrict__ tw, int b) {
-    auto at = [&](int k) {
-        float2 w = TW_SHARED ? tw[k] : __ldg(tw + k);
-        if (INV) w.y = -w.y;
-        return w;
-    };
+    auto at = [&](int k) { return TW_SHARED ? tw[k] : __ldg(tw + k); };
     const float2 lo[4] = {make_float2(1.f, 0.f), at(b), at(2 * b), at(3 * b)};
     const float2 hi[4] = {make_float2(1.f, 0.f), at(4 * b), at(8 * b), at(12 * b)};
 #pragma unroll
     for (int k = 1; k < 16; k++) {
         const int a = k & 3, c = k >> 2;
-        const float2 w = a == 0 ? hi[c] : (c == 0 ? lo[a] : cmul(lo[a], hi[c]));
-        v[k] = cmul(v[k], w);
+        if (a == 0 || c == 0) {
+            const float2 w = a == 0 ? hi[c] : lo[a];
+            v[k] = INV ? cmulc(v[k], w) : cmul(v[k], w);
+        } else {
+            const float2 w = INV ? cmul(lo[a], hi[c]) : cmul(hi[c], lo[a]);
+            v[k] = cmul(v[k], INV ? conjf2(w) : w);
+        }
     }
 }
 

@@ -10,9 +10,11 @@
 //            exchange + anisotropy + Zeeman + cavity B_rms Gamma (Sec. 2.1
 //            field terms, Eq. bcav), the LLG torque (Eq. llg), the RK
 //            bookkeeping, and block partials of the coupling sum
-//            X = V_c sum_i Ms_i m_i . B_rms,i (Eq. gammafinal).  The last block
-//            of each instance to finish reduces the partials in a fixed order
-//            and advances the cavity amplitude / step-size controller in FP64.
+//            X = V_c sum_i Ms_i m_i . B_rms,i (Eq. gammafinal).
+// The partials are reduced in a fixed order and the cavity amplitudes advanced
+// in FP64 by one extra block of the next x forward (scalar_block); at the end
+// of a Dormand-Prince attempt, whose decision the next x forward reads, and of
+// a call by the last x inverse block of the instance to finish.
 #include <math.h>
 
 #include "common.cuh"
@@ -29,7 +31,9 @@ namespace mq {
 // ---------------------------------------------------------------------------
 // FX: the fixed shape of the large grids (see xpass_fixed) at compile time.
 template <int L, bool FX>
-__global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(Plan P, Buffers Bf, StageArgs A) {
+__global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(
+    const __grid_constant__ Plan P, const __grid_constant__ Material mat, const __grid_constant__ Buffers Bf,
+    const __grid_constant__ StageArgs A) {
     constexpr bool F3 = xpass_f3(L);
     constexpr int NPT = F3 ? 16 : ColShape<L>::NPT, N1 = xpass_line_threads(L);
     constexpr int RF = xpass_rows(L);
@@ -37,11 +41,17 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(Pla
     const int b = A.inst0 + blockIdx.y;
     const InstState& st = Bf.st[b];
     if (stage_skips(st, A)) return;
+    if (blockIdx.x == 0) {
+        __shared__ double s_red[32 * (MAX_MODES + 3)];
+        __shared__ float s_redf[32];
+        scalar_block(P, mat, Bf, A, b, s_red, s_redf);
+        return;
+    }
     const int Rb = FX ? RF : P.R;
     const int nx = FX ? L : P.nx;
     const int px = FX ? 2 * L : P.px;
     const int nthr = FX ? 3 * RF * N1 : (int)blockDim.x;
-    const int row0 = blockIdx.x * Rb;
+    const int row0 = ((int)blockIdx.x - 1) * Rb;
     const int nr = FX ? RF : min(P.R, P.nrows - row0);
     const int ld = xpass_ld(Rb);
     const long long base = (long long)b * P.N + (long long)row0 * nx;
@@ -87,18 +97,21 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(Pla
         const int nl = 3 * Rb;
         const int line = F3 ? threadIdx.x / N1 : threadIdx.x % nl;
         const int j = F3 ? threadIdx.x % N1 : threadIdx.x / nl;
+        // threads beyond the lines (blocks of few rows) pass the barriers only
+        const bool act = FX || F3 || j < N1;
         float2 v[NPT];
 #pragma unroll
         for (int n2 = 0; n2 < NPT; n2++)
-            v[n2] = (!FX || n2 < NPT / 2) ? zs[(j + N1 * n2) * ld + line] : make_float2(0.f, 0.f);
+            v[n2] = act && (!FX || n2 < NPT / 2) ? zs[(j + N1 * n2) * ld + line] : make_float2(0.f, 0.f);
         if constexpr (F3) {
             col_fft3<L, false, false, XPASS_F3_PADS, 1>(v, zs, ld, line, j, Bf.tw, P.twn);
 #pragma unroll
             for (int i = 0; i < NPT; i++) zs[col3_out_row<L>(j, i) * ld + line] = v[i];
         } else {
-            col_fft<L, false, true>(v, zs, ld, line, j, stw, px);
+            col_fft<L, false, true>(v, zs, ld, line, j, stw, px, act);
+            if (act)
 #pragma unroll
-            for (int i = 0; i < NPT; i++) zs[col_out_row<L>(j, i) * ld + line] = v[i];
+                for (int i = 0; i < NPT; i++) zs[col_out_row<L>(j, i) * ld + line] = v[i];
         }
     }
     __syncthreads();
@@ -115,7 +128,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(Pla
             float2 E = make_float2(0.5f * (Zk.x + Zc.x), 0.5f * (Zk.y + Zc.y));
             float2 D = make_float2(0.5f * (Zk.x - Zc.x), 0.5f * (Zk.y - Zc.y));
             float2 wD = cmul(F3 ? __ldg(Bf.tw + k * tws) : stw[k], D);
-            X = make_float2(E.x + wD.y, E.y - wD.x);
+            X = make_float2(__fadd_rn(E.x, wD.y), __fsub_rn(E.y, wD.x));
         }
         return X;
     };
@@ -287,14 +300,27 @@ __global__ void k_set_dt(InstState* st, int B, double dt) {
 // ---------------------------------------------------------------------------
 // host-side launchers (called from the C ABI)
 // ---------------------------------------------------------------------------
-// Rows per x-pass block: R lines of 3 components times N1 = L / 32 threads
-// each, aiming at ~192 threads per block.
+// Most rows of an x-pass block: R rows of 3 lines times N1 threads each, 192
+// threads of the transform at most.
 int rows_per_block(int L, int nrows) {
     int n1 = xpass_line_threads(L);
     int R = 64 / n1;
     if (R < 1) R = 1;
     if (R > nrows) R = nrows;
     return R;
+}
+
+// Rows of an x-pass block, at most `most`: as few as keep the launch within
+// two blocks per SM.  A grid with fewer rows than that is bound by the latency
+// of one block (its rows go through the load, transform and store loops one
+// after the other), so it gets more, smaller blocks: a 32x32 film as one block
+// of 32 rows took 9.1 us in the x forward and 19.8 us in the x inverse, as 32
+// blocks of one row 3.2 and 6.2 us.  Measured at 1, 2 and 4 blocks per SM: a
+// 300x120x5 strip 1.42, 1.33 and 1.55 ms per 3 attempts, 16 films of 100x75
+// 4.13, 3.85 and 3.86 ms per 20 steps.
+int rows_within(int most, long long rows_total, int sms) {
+    long long R = (rows_total + 2LL * sms - 1) / (2LL * sms);
+    return R < 1 ? 1 : (R > most ? most : (int)R);
 }
 
 
@@ -309,20 +335,22 @@ size_t xfwd_smem(const Plan& P) {
 bool x_fits(const Plan& P) { return P.L <= 1024 && xthreads(P) <= 512 && xinv_smem(P) <= 200 * 1024; }
 
 
-cudaError_t launch_xfwd(const Plan& P, const Buffers& Bf, const StageArgs& A, int nb, cudaStream_t s) {
-    dim3 grid(P.nblk, nb);
+// One block more than the rows need per instance: the scalar block.
+cudaError_t launch_xfwd(const Plan& P, const Material& mat, const Buffers& Bf, const StageArgs& A, int nb,
+                        cudaStream_t s) {
+    dim3 grid(P.nblk + 1, nb);
     const int th = xthreads(P);
     const size_t sm = xfwd_smem(P);
     if (xpass_fixed(P)) {
         switch (P.L) {
-#define MMCQ_CASE(Lv) case Lv: return launch_chain(k_xfwd<Lv, true>, grid, th, sm, s, P, Bf, A);
+#define MMCQ_CASE(Lv) case Lv: return launch_chain(k_xfwd<Lv, true>, grid, th, sm, s, P, mat, Bf, A);
             MMCQ_XFIXED(MMCQ_CASE)
 #undef MMCQ_CASE
             default: break;
         }
     }
     switch (P.L) {
-#define MMCQ_CASE(Lv) case Lv: return launch_chain(k_xfwd<Lv, false>, grid, th, sm, s, P, Bf, A);
+#define MMCQ_CASE(Lv) case Lv: return launch_chain(k_xfwd<Lv, false>, grid, th, sm, s, P, mat, Bf, A);
         MMCQ_XCASES(MMCQ_CASE)
 #undef MMCQ_CASE
         default: return cudaErrorInvalidValue;

@@ -1,6 +1,6 @@
-// Device code shared by the stage kernels (stage.cu): Runge-Kutta
+// Device code shared by the stage kernels (stage.cu, xinv.cu): Runge-Kutta
 // tableaux, the per-cell field / torque / RK update, the FP64 block
-// reductions and the per-instance finisher.  Included by each translation
+// reductions and the per-instance scalar work.  Included by each translation
 // unit; constant-memory tables are per unit and filled by upload_tableaux().
 #pragma once
 
@@ -27,7 +27,7 @@ __device__ __forceinline__ float warp_max_f(float v) {
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_down_sync(0xffffffffu, v, o));
     return v;
 }
-// Fixed-shape block reductions (deterministic for a given blockDim).
+// Fixed-shape block reduction (deterministic for a given blockDim).
 static __device__ double block_sum_d(double v, double* red) {
     v = warp_sum_d(v);
     int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -42,150 +42,203 @@ static __device__ double block_sum_d(double v, double* red) {
     __syncthreads();
     return r;  // valid in thread 0
 }
-static __device__ float block_max_f(float v, float* red) {
-    v = warp_max_f(v);
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) red[w] = v;
-    __syncthreads();
-    int nw = (blockDim.x + 31) >> 5;
-    float r = 0.f;
-    if (w == 0) {
-        r = l < nw ? red[l] : 0.f;
-        r = warp_max_f(r);
+
+// Sums of the NQ doubles and the maximum of the float (with_max, uniform) of
+// every thread, in one block barrier for all of them: the results are valid
+// in thread 0.  `red` holds NQ rows and `redf` one row of 32 warp values; the
+// caller synchronises before they are written again.
+template <int NQ>
+static __device__ __forceinline__ void block_reduce(double (&v)[NQ], float& mx, bool with_max, double* red,
+                                                    float* redf) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int q = 0; q < NQ; q++) v[q] = warp_sum_d(v[q]);
+    if (with_max) mx = warp_max_f(mx);
+    if (l == 0) {
+#pragma unroll
+        for (int q = 0; q < NQ; q++) red[q * 32 + w] = v[q];
+        redf[w] = mx;
     }
     __syncthreads();
-    return r;
+    if (w == 0) {
+#pragma unroll
+        for (int q = 0; q < NQ; q++) v[q] = warp_sum_d(l < nw ? red[q * 32 + l] : 0.0);
+        if (with_max) mx = warp_max_f(l < nw ? redf[l] : 0.f);
+    }
 }
 
-// Gamma_k(t) from the P-mode accumulators, Eq. (gammadiscretefinal).
-static __device__ double gamma_p(const InstParams& ip, const InstState& s, int k, double tc, double hbar) {
-    double e = exp(-ip.kappa[k] * tc);
-    double sn, cs;
-    sincos(ip.wc[k] * tc, &sn, &cs);
+// Gamma_k from the P-mode accumulators, Eq. (gammadiscretefinal), with e =
+// exp(-kappa t), sn and cs the sine and cosine of omega t.
+static __device__ double gamma_p(const InstParams& ip, const InstState& s, int k, double e, double sn, double cs,
+                                 double hbar) {
     return e * cs * (ip.x0[k] - 2.0 * s.S[k] / hbar) - e * sn * (ip.p0[k] - 2.0 * s.C[k] / hbar);
 }
 
-// FP64 scalar work after the last block of an instance has finished a stage:
-// for every cavity mode k the amplitude (E-mode: d alpha_k/dt =
-// -(kappa_k + i omega_k) alpha_k + i X_k / hbar, Eq. eqmotionaclasical with
-// omega_c -> omega_c - i kappa) or the accumulators (P-mode, Eq. Sdiscrete /
-// Cdiscrete); then time, accept / reject and step size.  Xsum[k] holds the
-// coupling sums without V_c.
-static __device__ void finish_stage(const Plan& P, const Material& mat, const StageArgs& A, const InstParams& ip,
-                             InstState& s, const double* Xsum, float errmax, double* hist, int hcap, int* flags,
-                             const double* msum = nullptr, double* mhist = nullptr) {
-    const int k = A.stage;
-    const int K = A.kind;
-    const int nm = A.nmodes;
-    const double dt = s.dt;
-    for (int q = 0; q < nm; q++) {
-        const double X = Xsum[q] * mat.vc;
-        s.X[q] = X;
-        if (ip.cav_on[q] && A.mode == CAV_E) {
-            // derivative of alpha_q at this stage
-            s.ka_re[q][k] = -ip.kappa[q] * s.as_re[q] + ip.wc[q] * s.as_im[q];
-            s.ka_im[q][k] = -ip.kappa[q] * s.as_im[q] - ip.wc[q] * s.as_re[q] + X / mat.hbar;
-        }
-    }
-    const int nst = K == KIND_RK4 ? 4 : 7;
-    const bool last = k == nst - 1;
-    if (!last) {
-        // alpha of the next stage (DP45 stage 7 takes the 5th-order weights)
-        const bool to_b = (K == KIND_DP45 && k + 1 == 6);
-        for (int q = 0; q < nm; q++) {
-            if (!ip.cav_on[q] || A.mode != CAV_E) continue;
-            double re = s.a_re[q], im = s.a_im[q];
-            for (int j = 0; j <= k; j++) {
-                double w = to_b ? c_bd[1][j] : c_ad[K][k + 1][j];
-                re += dt * w * s.ka_re[q][j];
-                im += dt * w * s.ka_im[q][j];
-            }
-            s.as_re[q] = re;
-            s.as_im[q] = im;
-        }
-        if (K == KIND_DP45 && k == 0) s.have_k1 = 1;
-        return;
-    }
-    int accept = 1;
-    if (K == KIND_DP45) {
-        float tol = A.tol;
-        if (s.poison || !(errmax == errmax)) errmax = INFINITY;
-        accept = errmax <= tol;
-    }
-    if (accept) {
-        if (K == KIND_RK4) {
-            for (int q = 0; q < nm; q++) {
-                if (!ip.cav_on[q] || A.mode != CAV_E) continue;
-                double re = s.a_re[q], im = s.a_im[q];
-                for (int j = 0; j < 4; j++) {
-                    re += dt * c_bd[0][j] * s.ka_re[q][j];
-                    im += dt * c_bd[0][j] * s.ka_im[q][j];
-                }
-                s.a_re[q] = re; s.a_im[q] = im;
-            }
-        } else {
-            s.mcur ^= 1;
-            s.k1slot = s.k1slot == 0 ? 6 : 0;
-            for (int q = 0; q < nm; q++) {
-                if (!ip.cav_on[q] || A.mode != CAV_E) continue;
-                s.a_re[q] = s.as_re[q]; s.a_im[q] = s.as_im[q];   // alpha5
-                s.ka_re[q][0] = s.ka_re[q][6]; s.ka_im[q][0] = s.ka_im[q][6];
-            }
-            if (A.mode == CAV_P) s.have_k1 = 0;   // Gamma at t_n changes with S_n, C_n
-        }
-        s.t += dt;
-        s.tcav += dt;
-        s.nacc++;
-        if (s.nhist < hcap) hist[s.nhist] = dt;
-        else atomicOr(flags, FLAG_HIST_FULL);
-        s.nhist++;
-        if (A.record > 0 && msum && mhist && s.nacc % A.record == 0) {
-            if (s.nmh < hcap) {
-                double* e = mhist + 4 * s.nmh;
-                e[0] = s.t;
-                for (int c = 0; c < 3; c++) e[1 + c] = msum[c] * ip.inv_nmag;
-            } else {
-                atomicOr(flags, FLAG_HIST_FULL);
-            }
-            s.nmh++;
-        }
-        if (A.mode == CAV_P) {
-            for (int q = 0; q < nm; q++) {
-                if (!ip.cav_on[q]) continue;
-                double e = exp(ip.kappa[q] * s.tcav), sn, cs;
-                sincos(ip.wc[q] * s.tcav, &sn, &cs);
-                s.S[q] += e * sn * s.X[q] * dt;
-                s.C[q] += e * cs * s.X[q] * dt;
-            }
-        }
-    } else {
-        s.nrej++;
-    }
-    if (K == KIND_DP45) {
-        double err = (double)errmax;
-        double f = err > 0.0 ? 0.9 * pow((double)A.tol / err, 0.2) : 5.0;
-        if (!(f == f)) f = 0.2;
-        f = fmin(5.0, fmax(0.2, f));
-        double nd = dt * f;
-        s.err = err;
-        s.poison = 0;
-        if (s.t_end > 0.0) {
-            if (s.t >= s.t_end * (1.0 - 1e-14)) s.done = 1;
-            else if (s.t + nd > s.t_end) nd = s.t_end - s.t;
-        }
-        if (nd < 1e-20 && !s.done) { atomicOr(flags, FLAG_DT_UNDERFLOW); s.done = 1; }
-        s.dt = nd;
-    }
-    for (int q = 0; q < nm; q++) {
-        if (!ip.cav_on[q] || A.mode != CAV_E) continue;
-        if (K == KIND_DP45) {
-            s.as_re[q] = s.a_re[q] + s.dt * c_ad[1][1][0] * s.ka_re[q][0];
-            s.as_im[q] = s.a_im[q] + s.dt * c_ad[1][1][0] * s.ka_im[q][0];
-        } else {
-            s.as_re[q] = s.a_re[q]; s.as_im[q] = s.a_im[q];
-        }
-    }
+// X / hbar from the product with the reciprocal and one correction step (the
+// division's own code is a long dependent chain on this part's FP64 pipe); the
+// division itself where that is not finite.
+__device__ __forceinline__ double over_hbar(double X, const Material& mat) {
+    const double q = X * mat.inv_hbar;
+    const double r = fma(fma(-q, mat.hbar, X), mat.inv_hbar, q);
+    return fabs(r) <= 1e300 ? r : X / mat.hbar;
 }
+
+// FP64 scalar work of one instance at the end of stage k, by one warp: lane
+// q < A.nmodes does mode q's arithmetic -- the amplitude (E-mode: d alpha_k/dt
+// = -(kappa_k + i omega_k) alpha_k + i X_k / hbar, Eq. eqmotionaclasical with
+// omega_c -> omega_c - i kappa) or the accumulators (P-mode, Eq. Sdiscrete /
+// Cdiscrete) -- and lane 0 also time, accept / reject and step size.
+// load(): everything that does not depend on this stage's coupling sums: the
+// state (independent loads) and the Runge-Kutta sums over the earlier stages,
+// to run while the partials are on their way.  finish(): the rest, a few
+// dependent FP64 operations.  (One thread that copied the 750-byte state to its
+// stack and then did every mode took 4.7 us of a 20 us x inverse.)
+struct StageFinish {
+    double dt, tcav;
+    double re, im;       // E-mode: alpha_q plus the terms of the stages before k
+    double ar, ai;       // E-mode: alpha_q of stage k
+    double dr, di;       // E-mode: its derivative without X / hbar
+    double w;            // dt times the weight of stage k
+    double k0r, k0i;     // E-mode: derivative of stage 1
+    bool cav, amp, last;
+
+    __device__ __forceinline__ void load(const StageArgs& A, int k, const InstParams& ip, const InstState& s) {
+        const int q = threadIdx.x & 31, K = A.kind;
+        cav = q < A.nmodes && ip.cav_on[q < MAX_MODES ? q : 0] != 0;
+        amp = cav && A.mode == CAV_E;
+        last = k == (K == KIND_RK4 ? 3 : 6);
+        dt = s.dt;
+        tcav = s.tcav;
+        re = im = ar = ai = dr = di = w = k0r = k0i = 0.0;
+        if (!amp) return;
+        double kr[MAX_STAGES - 1], ki[MAX_STAGES - 1];
+#pragma unroll
+        for (int j = 0; j < MAX_STAGES - 1; j++) {
+            kr[j] = j < k ? s.ka_re[q][j] : 0.0;
+            ki[j] = j < k ? s.ka_im[q][j] : 0.0;
+        }
+        re = s.a_re[q];
+        im = s.a_im[q];
+        ar = s.as_re[q];
+        ai = s.as_im[q];
+        k0r = kr[0];
+        k0i = ki[0];
+        dr = -ip.kappa[q] * ar + ip.wc[q] * ai;
+        di = -ip.kappa[q] * ai - ip.wc[q] * ar;
+        // weights of the next stage (DP45 stage 7: the 5th-order ones), or of
+        // the step (RK4's last stage; DP45's last is already its alpha5)
+        if (last && K == KIND_DP45) return;
+        const double* c = last || (K == KIND_DP45 && k == 5) ? c_bd[K] : c_ad[K][k + 1];
+#pragma unroll
+        for (int j = 0; j < MAX_STAGES - 1; j++)
+            if (j < k) {
+                re += dt * c[j] * kr[j];
+                im += dt * c[j] * ki[j];
+            }
+        w = dt * c[k];
+    }
+
+    // Xsum: the mode's coupling sum without V_c (lane q); errmax uniform over
+    // the warp; msum read by lane 0; trig[0..2][q] (P-mode, last stage):
+    // exp(kappa t), sin and cos of omega t at the end of the step.
+    __device__ __forceinline__ void finish(const Material& mat, const StageArgs& A, int k, const InstParams& ip,
+                                           InstState& s, double Xsum, float errmax, double* hist, int hcap, int* flags,
+                                           const double* msum, double* mhist, const double (*trig)[MAX_MODES]) {
+        const int q = threadIdx.x & 31, K = A.kind;
+        const double X = Xsum * mat.vc;
+        if (q < A.nmodes) s.X[q] = X;
+        if (amp) {
+            di += over_hbar(X, mat);
+            s.ka_re[q][k] = dr;
+            s.ka_im[q][k] = di;
+            re += w * dr;
+            im += w * di;
+        }
+        if (!last) {
+            if (amp) {
+                s.as_re[q] = ar = re;
+                s.as_im[q] = ai = im;
+            }
+            if (q == 0 && K == KIND_DP45 && k == 0) s.have_k1 = 1;
+            return;
+        }
+        bool accept = true;
+        double nd = dt;                     // next step length
+        if (K == KIND_DP45) {
+            if (s.poison || !(errmax == errmax)) errmax = INFINITY;
+            accept = errmax <= A.tol;
+            const double err = (double)errmax;
+            double f = err > 0.0 ? 0.9 * pow((double)A.tol / err, 0.2) : 5.0;
+            if (!(f == f)) f = 0.2;
+            f = fmin(5.0, fmax(0.2, f));
+            nd = dt * f;
+            const double t = accept ? s.t + dt : s.t, te = s.t_end;
+            bool done = false;
+            if (te > 0.0) {
+                if (t >= te * (1.0 - 1e-14)) done = true;
+                else if (t + nd > te) nd = te - t;
+            }
+            if (nd < 1e-20 && !done) {
+                if (q == 0) atomicOr(flags, FLAG_DT_UNDERFLOW);
+                done = true;
+            }
+            __syncwarp();                   // every lane has read the state
+            if (q == 0) {
+                s.err = err;
+                s.poison = 0;
+                if (done) s.done = 1;
+                s.dt = nd;
+            }
+        }
+        if (amp) {
+            if (K == KIND_DP45 && accept) {
+                re = ar;                    // alpha5
+                im = ai;
+                s.ka_re[q][0] = k0r = dr;
+                s.ka_im[q][0] = k0i = di;
+            }
+            if (accept) {
+                s.a_re[q] = re;
+                s.a_im[q] = im;
+            }
+            // amplitude of the stage evaluated next
+            ar = K == KIND_DP45 ? re + nd * c_ad[1][1][0] * k0r : re;
+            ai = K == KIND_DP45 ? im + nd * c_ad[1][1][0] * k0i : im;
+            s.as_re[q] = ar;
+            s.as_im[q] = ai;
+        } else if (cav && accept) {
+            s.S[q] += trig[0][q] * trig[1][q] * X * dt;
+            s.C[q] += trig[0][q] * trig[2][q] * X * dt;
+        }
+        if (q == 0) {
+            if (accept) {
+                if (K == KIND_DP45) {
+                    s.mcur ^= 1;
+                    s.k1slot = s.k1slot == 0 ? 6 : 0;
+                    if (A.mode == CAV_P) s.have_k1 = 0;   // Gamma at t_n changes with S_n, C_n
+                }
+                s.t += dt;
+                s.tcav = tcav + dt;
+                s.nacc++;
+                if (s.nhist < hcap) hist[s.nhist] = dt;
+                else atomicOr(flags, FLAG_HIST_FULL);
+                s.nhist++;
+                if (A.record > 0 && mhist && s.nacc % A.record == 0) {
+                    if (s.nmh < hcap) {
+                        double* e = mhist + 4 * s.nmh;
+                        e[0] = s.t;
+                        for (int c = 0; c < 3; c++) e[1 + c] = msum[c] * ip.inv_nmag;
+                    } else {
+                        atomicOr(flags, FLAG_HIST_FULL);
+                    }
+                    s.nmh++;
+                }
+            } else {
+                s.nrej++;
+            }
+        }
+    }
+};
 
 static void upload_tableaux() {
     float af[2][MAX_STAGES][MAX_STAGES] = {};
@@ -310,16 +363,16 @@ struct CellUpdate {
     // fb_: first cell of the launch's first instance; a field evaluation writes
     // fout[i - fb_], so a launch over several instances fills [instances][N]
     __device__ __forceinline__ void init(const Buffers& Bf, const StageArgs& A, const InstState& st,
-                                         const InstParams& ip, const double* gam, float drive, long long cb_,
+                                         const InstParams& ip, const StageScalars& sc, long long cb_,
                                          long long fb_) {
         nm = NM == 1 ? 1 : A.nmodes;
 #pragma unroll
         for (int q = 0; q < NM; q++) {
-            G[q] = (float)gam[q];
+            G[q] = sc.gamma[q];
             bs[q] = (float)ip.brms_scale[q];
             on[q] = q < nm && ip.cav_on[q] != 0;
         }
-        D = drive;
+        D = sc.drive;
         dt = (float)st.dt;
         bex = (float)ip.bext[0]; bey = (float)ip.bext[1]; bez = (float)ip.bext[2];
         want_demag = A.terms & 1; want_exch = A.terms & 2;
@@ -427,23 +480,147 @@ static __device__ double drive_factor(const StageArgs& A, const InstParams& ip, 
     return ip.drv_amp * (x == 0.0 ? 1.0 : sin(x) / x);
 }
 
-// Gamma_k(t) for the stage of this launch (E-mode: 2 Re alpha_k of the stage;
-// P-mode: Eq. gammadiscretefinal at the stage time).
-static __device__ double stage_gamma(const StageArgs& A, const InstParams& ip, const InstState& st,
-                                     const Material& mat, int k) {
-    if (!ip.cav_on[k]) return 0.0;
-    if (A.mode == CAV_E) return 2.0 * (A.field_only ? st.a_re[k] : st.as_re[k]);
-    return gamma_p(ip, st, k, st.tcav + (A.field_only ? 0.0 : c_cd[A.kind][A.stage] * st.dt), mat.hbar);
+// Whether this is the last stage of a step.
+__device__ __forceinline__ bool stage_last(const StageArgs& A) { return A.stage == (A.kind == KIND_RK4 ? 3 : 6); }
+
+// Whether a launch records the spatial average of the state being accepted:
+// the last stage of a step with recording on (stage k).
+__device__ __forceinline__ bool stage_records(const StageArgs& A, int k) {
+    return A.record > 0 && k == (A.kind == KIND_RK4 ? 3 : 6);
 }
 
-// Block partials of X_k and of the DP45 error; the last block of the instance
-// to arrive reduces all partials in a fixed order and runs finish_stage.
-// `nparts` = blocks per instance, `part` = this block's index among them.
-// Partials of mode k live at xpart[(k B + b) nparts + part].
+// All partials of instance b of stage k reduced in a fixed order by this
+// block, then the scalar work of that stage, by warp 0: on return f holds the
+// lane's mode.  trig as for StageFinish::finish, in shared memory, written by
+// other warps before the call.
+static __device__ __forceinline__ void finish_instance(const Plan& P, const Material& mat, const Buffers& Bf,
+                                                       const StageArgs& A, int b, int k, StageFinish& f,
+                                                       double* s_red, float* s_redf,
+                                                       const double (*trig)[MAX_MODES]) {
+    const int n = A.nparts;
+    const long long pb = (long long)b * n;
+    const bool rec = stage_records(A, k), dp_last = A.kind == KIND_DP45 && k == 6;
+    const InstParams& ip = Bf.ip[b];
+    InstState& st = Bf.st[b];
+    double v[MAX_MODES + 3];
+#pragma unroll
+    for (int q = 0; q < MAX_MODES + 3; q++) v[q] = 0.0;
+    float em = 0.f;
+    const long long ms = (long long)P.B * n;
+    if (A.nmodes == 1 && !rec) {
+        double x[1] = {0.0};
+        for (int r = threadIdx.x; r < n; r += blockDim.x) {
+            x[0] += __ldcg(Bf.xpart + pb + r);
+            if (dp_last) em = fmaxf(em, __ldcg(Bf.epart + pb + r));
+        }
+        if (threadIdx.x < 32) f.load(A, k, ip, st);
+        block_reduce<1>(x, em, dp_last, s_red, s_redf);
+        v[0] = x[0];
+    } else {
+        for (int r = threadIdx.x; r < n; r += blockDim.x) {
+#pragma unroll
+            for (int q = 0; q < MAX_MODES; q++)
+                if (q < A.nmodes) v[q] += __ldcg(Bf.xpart + q * ms + pb + r);
+            if (dp_last) em = fmaxf(em, __ldcg(Bf.epart + pb + r));
+            if (rec)
+                for (int c = 0; c < 3; c++) v[MAX_MODES + c] += __ldcg(Bf.mpart + 3 * (pb + r) + c);
+        }
+        if (threadIdx.x < 32) f.load(A, k, ip, st);
+        block_reduce<MAX_MODES + 3>(v, em, dp_last, s_red, s_redf);
+    }
+    if (threadIdx.x < 32) {
+        double x = v[0];
+        if (A.nmodes > 1) {
+#pragma unroll
+            for (int q = 0; q < MAX_MODES; q++) {
+                const double w = __shfl_sync(0xffffffffu, v[q], 0);
+                if (threadIdx.x == q) x = w;
+            }
+        }
+        em = __shfl_sync(0xffffffffu, em, 0);
+        f.finish(mat, A, k, ip, st, x, em, Bf.hist + (long long)b * Bf.hcap, Bf.hcap, Bf.flags, v + MAX_MODES,
+                 rec ? Bf.mhist + 4LL * b * Bf.hcap : nullptr, trig);
+    }
+}
+
+// exp(sign kappa t), sin and cos of omega t of mode q at cavity time t.
+static __device__ __noinline__ void mode_trig(const InstParams& ip, int q, double sign, double t,
+                                              double (*trig)[MAX_MODES]) {
+    double sn, cs;
+    sincos(ip.wc[q] * t, &sn, &cs);
+    trig[0][q] = exp(sign * ip.kappa[q] * t);
+    trig[1][q] = sn;
+    trig[2][q] = cs;
+}
+
+// The scalar block of instance b in an x forward (one extra block per
+// instance, running beside the row blocks, which need none of what it writes):
+// the scalar work the previous stage left (A.fin_prev), then Gamma_k and the
+// excitation of this stage for the x inverse that follows.  So neither the
+// end of one x inverse nor the start of the next waits for FP64 arithmetic
+// (P-mode: an exponential and a sine of each mode in every block, 9 us of a
+// 17 us x inverse of a 50^3 sphere with two modes).
+static __device__ __noinline__ void scalar_block(const Plan& P, const Material& mat, const Buffers& Bf,
+                                                 const StageArgs& A, int b, double* s_red, float* s_redf) {
+    __shared__ double s_end[3][MAX_MODES], s_now[3][MAX_MODES];
+    const InstParams& ip = Bf.ip[b];
+    const InstState& st = Bf.st[b];
+    // a Dormand-Prince stage 1 that was skipped (kept from the last attempt)
+    // has nothing to finish
+    const bool kept = A.kind == KIND_DP45 && A.fin_prev == 0 && st.have_k1;
+    const bool fin = A.fin_prev >= 0 && !kept;
+    const bool step_end = fin && A.kind == KIND_RK4 && A.fin_prev == 3;
+    const double dt = st.dt;
+    const double t_end = st.tcav + (step_end ? dt : 0.0);
+    const double t_now = t_end + (A.field_only ? 0.0 : c_cd[A.kind][A.stage] * dt);
+    if (threadIdx.x >= 32 && threadIdx.x < 32 + A.nmodes && A.mode == CAV_P) {
+        // beside the loads and the reduction of warp 0
+        const int q = threadIdx.x - 32;
+        if (ip.cav_on[q]) {
+            if (step_end) mode_trig(ip, q, 1.0, t_end, s_end);
+            mode_trig(ip, q, -1.0, t_now, s_now);
+        }
+    }
+    __syncthreads();        // (and every thread has read the state that warp 0 changes)
+    StageFinish f;
+    f.ar = 0.0;
+    if (fin) finish_instance(P, mat, Bf, A, b, A.fin_prev, f, s_red, s_redf, s_end);
+    if (threadIdx.x >= 32) return;
+    __syncwarp();
+    const int q = threadIdx.x;
+    if (q < A.nmodes) {
+        double G = 0.0;
+        if (ip.cav_on[q])
+            G = A.mode == CAV_P ? gamma_p(ip, st, q, s_now[0][q], s_now[1][q], s_now[2][q], mat.hbar)
+                                : 2.0 * (A.field_only ? st.a_re[q] : (fin ? f.ar : st.as_re[q]));
+        Bf.sc[b].gamma[q] = (float)G;
+    }
+    if (q == MAX_MODES) Bf.sc[b].drive = (float)drive_factor(A, ip, st);
+}
+
+// The scalar work of this stage, by the last x inverse block to finish.
+static __device__ __noinline__ void finish_here(const Plan& P, const Material& mat, const Buffers& Bf,
+                                                const StageArgs& A, int b, double* s_red, float* s_redf) {
+    __shared__ double s_end[3][MAX_MODES];
+    if (threadIdx.x >= 32 && threadIdx.x < 32 + A.nmodes && A.mode == CAV_P && stage_last(A)) {
+        const int q = threadIdx.x - 32;
+        const InstState& st = Bf.st[b];
+        if (Bf.ip[b].cav_on[q]) mode_trig(Bf.ip[b], q, 1.0, st.tcav + st.dt, s_end);
+    }
+    __syncthreads();
+    StageFinish f;
+    finish_instance(P, mat, Bf, A, b, A.stage, f, s_red, s_redf, s_end);
+}
+
+// End of an x inverse block: its partials of X_k, of the DP45 error (last
+// stage) and of the recorded average.  With A.fin_here the last block of the
+// instance to arrive finishes the stage; otherwise the scalar block of the
+// next x forward does.  `part` = this block's index among A.nparts.
 template <bool REC, int NM>
-static __device__ void stage_epilogue(const Plan& P, const Material& mat, const Buffers& Bf, const StageArgs& A,
-                                      int b, int part, int nparts, const double (&xacc)[NM], float emax, bool bad,
-                                      double* s_red, float* s_redf, int* s_last, const double* macc) {
+static __device__ __forceinline__ void stage_epilogue(const Plan& P, const Material& mat, const Buffers& Bf,
+                                                      const StageArgs& A, int b, int part, const double (&xacc)[NM],
+                                                      float emax, bool bad, double* s_red, float* s_redf, int* s_last,
+                                                      const double* macc) {
     // RK4: a non-finite torque is an error.  DP45: it marks the attempt, which
     // is then rejected with the smallest step factor (an overflowing trial
     // step); a state that stays non-finite ends in step-size underflow.
@@ -451,54 +628,36 @@ static __device__ void stage_epilogue(const Plan& P, const Material& mat, const 
         if (A.kind == KIND_DP45) atomicOr(&Bf.st[b].poison, 1);
         else atomicOr(Bf.flags, FLAG_NAN);
     }
-    const int nm = NM == 1 ? 1 : A.nmodes;
-    double xb[NM];
+    const int nparts = A.nparts;
+    const bool dp_last = A.kind == KIND_DP45 && A.stage == 6;
+    constexpr int NQ = NM + (REC ? 3 : 0);
+    double v[NQ];
 #pragma unroll
-    for (int q = 0; q < NM; q++) xb[q] = q < nm ? block_sum_d(xacc[q], s_red) : 0.0;
-    float eb = block_max_f(emax, s_redf);
+    for (int q = 0; q < NM; q++) v[q] = xacc[q];
+    if constexpr (REC)
+        for (int c = 0; c < 3; c++) v[NM + c] = macc[c];
+    block_reduce<NQ>(v, emax, dp_last, s_red, s_redf);
     const long long pb = (long long)b * nparts;
-    double mb[3] = {0.0, 0.0, 0.0};
-    if (REC)
-        for (int c = 0; c < 3; c++) mb[c] = block_sum_d(macc[c], s_red);
     if (threadIdx.x == 0) {
+        const int nm = NM == 1 ? 1 : A.nmodes;
 #pragma unroll
         for (int q = 0; q < NM; q++)
-            if (q < nm) Bf.xpart[((long long)q * P.B + b) * nparts + part] = xb[q];
-        Bf.epart[pb + part] = eb;
-        if (REC)
-            for (int c = 0; c < 3; c++) Bf.mpart[3 * (pb + part) + c] = mb[c];
-        __threadfence();
-        unsigned prev = atomicAdd(Bf.counter + b, 1u);
-        *s_last = prev == (unsigned)(nparts - 1);
+            if (q < nm) Bf.xpart[((long long)q * P.B + b) * nparts + part] = v[q];
+        if (dp_last) Bf.epart[pb + part] = emax;
+        if constexpr (REC)
+            for (int c = 0; c < 3; c++) Bf.mpart[3 * (pb + part) + c] = v[NM + c];
+        if (A.fin_here) {
+            __threadfence();
+            unsigned prev = atomicAdd(Bf.counter + b, 1u);
+            *s_last = prev == (unsigned)(nparts - 1);
+        }
     }
+    if (!A.fin_here) return;
     __syncthreads();
     if (!*s_last) return;
     __threadfence();
-    double xs[MAX_MODES] = {0.0, 0.0, 0.0, 0.0};
-    for (int q = 0; q < nm; q++) {
-        double v = 0.0;
-        const double* xp = Bf.xpart + ((long long)q * P.B + b) * nparts;
-        for (int r = threadIdx.x; r < nparts; r += blockDim.x) v += __ldcg(xp + r);
-        xs[q] = block_sum_d(v, s_red);
-    }
-    float em = 0.f;
-    for (int r = threadIdx.x; r < nparts; r += blockDim.x) em = fmaxf(em, __ldcg(Bf.epart + pb + r));
-    em = block_max_f(em, s_redf);
-    double msum[3] = {0.0, 0.0, 0.0};
-    if (REC) {
-        for (int c = 0; c < 3; c++) {
-            double v = 0.0;
-            for (int r = threadIdx.x; r < nparts; r += blockDim.x) v += __ldcg(Bf.mpart + 3 * (pb + r) + c);
-            msum[c] = block_sum_d(v, s_red);
-        }
-    }
-    if (threadIdx.x == 0) {
-        InstState ns = Bf.st[b];
-        finish_stage(P, mat, A, Bf.ip[b], ns, xs, em, Bf.hist + (long long)b * Bf.hcap, Bf.hcap, Bf.flags,
-                     REC ? msum : nullptr, REC ? Bf.mhist + 4LL * b * Bf.hcap : nullptr);
-        Bf.st[b] = ns;
-        Bf.counter[b] = 0u;
-    }
+    if (threadIdx.x == 0) Bf.counter[b] = 0u;
+    finish_here(P, mat, Bf, A, b, s_red, s_redf);
 }
 
 }  // namespace mq

@@ -4,9 +4,10 @@
 // excitation) + cavity sum_k B_rms,k Gamma_k (Sec. 2.1 field terms, Eq. bcav),
 // the LLG torque (Eq. llg), the RK bookkeeping, and block partials of the
 // coupling sums X_k = V_c sum_i Ms_i m_i . B_rms,k,i (Eq. gammafinal): each
-// cell's FP32 product promoted and added in FP64.  The last block of each
-// instance to finish reduces the partials in a fixed order and advances the
-// cavity amplitudes and the step-size controller in FP64.
+// cell's FP32 product promoted and added in FP64.  The partials are reduced in
+// a fixed order, and the cavity amplitudes and the step-size controller
+// advanced in FP64, by the scalar block of the next x forward or, at the end
+// of an attempt or of a call, by the instance's last block to finish.
 #include <math.h>
 
 #include "common.cuh"
@@ -24,10 +25,10 @@ namespace mq {
 template <int L, int N1>
 __device__ __forceinline__ float2 unpack_twiddle(const float2* __restrict__ tw, int twstep, int j, int n2) {
     if constexpr (32 * N1 == 2 * L) {
-        const float2 wj = twiddle(tw, j * twstep, true);
-        return n2 == 0 ? wj : cmul(wj, conjf2(c_tw32[n2]));
+        const float2 wj = conjf2(__ldg(tw + j * twstep));
+        return n2 == 0 ? wj : cmulc(wj, c_tw32[n2]);
     } else {
-        return twiddle(tw, (j + N1 * n2) * twstep, true);
+        return conjf2(__ldg(tw + (j + N1 * n2) * twstep));
     }
 }
 
@@ -111,15 +112,15 @@ __device__ __forceinline__ void xinv_cells(const Plan& P, const Material& mat, c
 // FX: the fixed shape of the large grids (rows of nx = L cells, XPASS_ROWS(L)
 // rows per block with none left over, tiles of 8 kx columns) at compile time.
 template <int L, bool REC, int NM, bool FX>
-__global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(Plan P, Material mat, Buffers Bf, StageArgs A) {
+__global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(
+    const __grid_constant__ Plan P, const __grid_constant__ Material mat, const __grid_constant__ Buffers Bf,
+    const __grid_constant__ StageArgs A) {
     constexpr bool F3 = xpass_f3(L);
     constexpr int NPT = F3 ? 16 : ColShape<L>::NPT, N1 = xpass_line_threads(L);
     constexpr int RF = xpass_rows(L);
     extern __shared__ float2 sm[];
-    __shared__ double s_red[32];
+    __shared__ double s_red[32 * (MAX_MODES + 3)];
     __shared__ float s_redf[32];
-    __shared__ double s_gamma[NM];
-    __shared__ float s_drive;
     __shared__ int s_last;
     __shared__ int2 s_yz[64];                          // rows per block <= 64
     const int b = A.inst0 + blockIdx.y;
@@ -204,10 +205,6 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(Pla
     // the block's own rows of m are read in the cell loop (through L1, which
     // then serves the x and y neighbours as well)
     if (threadIdx.x == 0) prefetch_l2(msrc + base, (unsigned)(nr * nx * sizeof(float4)));
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < NM; q++) s_gamma[q] = stage_gamma(A, ip, st, mat, q);
-        s_drive = (float)drive_factor(A, ip, st);
-    }
     cp_async_wait_all();
     __syncthreads();
     const int twstep = P.twn / P.px;
@@ -217,6 +214,9 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(Pla
         const int nl = 3 * Rb;
         const int line = F3 ? threadIdx.x / N1 : threadIdx.x % nl;
         const int j = F3 ? threadIdx.x % N1 : threadIdx.x / nl;
+        // blocks of few rows have threads beyond the transform's lines, for
+        // the cells: they pass its barriers only
+        const bool act = FX || F3 || j < N1;
         // the C2R unpack done as the transform loads its points (k = j + N1 n2):
         // Z[k] = (X[k] + conj X[L-k]) + i e^{+2 pi i k / px} (X[k] - conj X[L-k]).
         // Every thread reads before the transform's first barrier, and no
@@ -225,26 +225,28 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(Pla
 #pragma unroll
         for (int n2 = 0; n2 < NPT; n2++) {
             const int k = j + N1 * n2;
+            if (!act) { v[n2] = make_float2(0.f, 0.f); continue; }
             const float2 a = xs[k * ld + line], bq = xs[(L - k) * ld + line];
             const float2 ca = conjf2(bq);
             const float2 sum = cadd(a, ca), dif = csub(a, ca);
             const float2 wd = cmul(unpack_twiddle<L, N1>(Bf.tw, twstep, j, n2), dif);
-            v[n2] = make_float2(sum.x - wd.y, sum.y + wd.x);   // sum + i wd
+            v[n2] = make_float2(__fsub_rn(sum.x, wd.y), __fadd_rn(sum.y, wd.x));   // sum + i wd
         }
         if constexpr (F3) {
             col_fft3<L, true, false, XPASS_F3_PADS, 1>(v, xs, ld, line, j, Bf.tw, P.twn);
 #pragma unroll
             for (int i = 0; i < NPT; i++) xs[col3_out_row<L>(j, i) * ld + line] = v[i];
         } else {
-            col_fft<L, true>(v, xs, ld, line, j, Bf.tw, P.twn);
+            col_fft<L, true>(v, xs, ld, line, j, Bf.tw, P.twn, act);
+            if (act)
 #pragma unroll
-            for (int i = 0; i < NPT; i++) xs[col_out_row<L>(j, i) * ld + line] = v[i];
+                for (int i = 0; i < NPT; i++) xs[col_out_row<L>(j, i) * ld + line] = v[i];
         }
     }
     __syncthreads();
 
     CellUpdate<NM> cu;
-    cu.init(Bf, A, st, ip, s_gamma, s_drive, cb, (long long)A.inst0 * P.N);
+    cu.init(Bf, A, st, ip, Bf.sc[b], cb, (long long)A.inst0 * P.N);
     double xacc[NM];
 #pragma unroll
     for (int q = 0; q < NM; q++) xacc[q] = 0.0;
@@ -253,7 +255,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(Pla
     bool bad = false;
     xinv_cells<NM, REC>(P, mat, Bf, cu, xs, ld, msrc, base, nx, nr, nthr, s_yz, xacc, macc, emax, bad);
     if (A.field_only) return;
-    stage_epilogue<REC, NM>(P, mat, Bf, A, b, blockIdx.x, P.nblk, xacc, emax, bad, s_red, s_redf, &s_last, macc);
+    stage_epilogue<REC, NM>(P, mat, Bf, A, b, blockIdx.x, xacc, emax, bad, s_red, s_redf, &s_last, macc);
 }
 
 // ---------------------------------------------------------------------------
@@ -277,17 +279,15 @@ static int g_sms = 0;                                        // SMs of the devic
 __device__ __forceinline__ int xpipe_land(int k, int c) { return 24 * (k >> 3) + 8 * c + (k & 7); }
 
 template <bool REC, int NM, bool FX>
-__global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(Plan P, Material mat, Buffers Bf,
-                                                                           StageArgs A,
-                                                                           const __grid_constant__ TensorMap tm) {
+__global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(
+    const __grid_constant__ Plan P, const __grid_constant__ Material mat, const __grid_constant__ Buffers Bf,
+    const __grid_constant__ StageArgs A, const __grid_constant__ TensorMap tm) {
     constexpr int L = 1024, N1 = 64, NPT = 16, ld = 3;
     extern __shared__ __align__(128) float2 sm_raw[];  // [2][XPIPE_BUF] from the first 128-byte boundary
     float2* sm = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(sm_raw) + 127) & ~(uintptr_t)127);
     __shared__ __align__(8) unsigned long long s_bar[2];
-    __shared__ double s_red[32];
+    __shared__ double s_red[32 * (MAX_MODES + 3)];
     __shared__ float s_redf[32];
-    __shared__ double s_gamma[NM];
-    __shared__ float s_drive;
     __shared__ int s_last;
     __shared__ int2 s_yz[1];
     const int b = A.inst0 + blockIdx.y;
@@ -323,14 +323,12 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(Plan 
         mbar_init(&s_bar[0], 1);
         mbar_init(&s_bar[1], 1);
         fence_proxy_async();
-        for (int q = 0; q < NM; q++) s_gamma[q] = stage_gamma(A, ip, st, mat, q);
-        s_drive = (float)drive_factor(A, ip, st);
     }
     __syncthreads();
     if (threadIdx.x == 0 && (int)blockIdx.x < P.nrows) issue(zfast_row(P, blockIdx.x), 0);
 
     CellUpdate<NM> cu;
-    cu.init(Bf, A, st, ip, s_gamma, s_drive, cb, (long long)A.inst0 * P.N);
+    cu.init(Bf, A, st, ip, Bf.sc[b], cb, (long long)A.inst0 * P.N);
     double xacc[NM];
 #pragma unroll
     for (int q = 0; q < NM; q++) xacc[q] = 0.0;
@@ -373,7 +371,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(Plan 
                 const float2 ca = conjf2(bq);
                 const float2 sum = cadd(a, ca), dif = csub(a, ca);
                 const float2 wd = cmul(unpack_twiddle<L, N1>(Bf.tw, twstep, j, n2), dif);
-                v[n2] = make_float2(sum.x - wd.y, sum.y + wd.x);
+                v[n2] = make_float2(__fsub_rn(sum.x, wd.y), __fadd_rn(sum.y, wd.x));
             }
             // (the transform's first barrier comes before its first store into xs)
             col_fft3<L, true, false, XPASS_F3_PADS, 1>(v, xs, ld, line, j, Bf.tw, P.twn);
@@ -386,7 +384,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(Plan 
         __syncthreads();   // buffer q and s_yz are rewritten by the next rows
     }
     if (A.field_only) return;
-    stage_epilogue<REC, NM>(P, mat, Bf, A, b, blockIdx.x, gridDim.x, xacc, emax, bad, s_red, s_redf, &s_last, macc);
+    stage_epilogue<REC, NM>(P, mat, Bf, A, b, blockIdx.x, xacc, emax, bad, s_red, s_redf, &s_last, macc);
 }
 
 // Whether the pipelined row kernel applies (see k_xinv_pipe) with this map.
@@ -394,13 +392,22 @@ static bool xpipe_applies(const Plan& P, const Buffers& Bf, const SpecMap* map) 
     return map && map->valid && map->base == Bf.spec && P.L == 1024 && P.TX == 8 && P.R == 1 && P.NT <= 256;
 }
 
+// persistent: XPIPE_BLOCKS per SM spread over the instances of the launch
+static int xpipe_blocks(const Plan& P, int nb) {
+    int per = (XPIPE_BLOCKS * g_sms + nb - 1) / nb;
+    if (per > P.nrows) per = P.nrows;
+    return per < 1 ? 1 : per;
+}
+
+// Blocks (and partials) per instance of an x inverse launch over nb instances.
+int xinv_parts(const Plan& P, const Buffers& Bf, int nb, const SpecMap* map, const Tune* T) {
+    return xpipe_applies(P, Bf, map) && (!T || T->x_pipe != 0) ? xpipe_blocks(P, nb) : P.nblk;
+}
+
 template <bool REC, int NM>
 static cudaError_t launch_xpipe(const Plan& P, const Material& mat, const Buffers& Bf, const StageArgs& A, int nb,
                          const SpecMap* map, cudaStream_t s) {
-    // persistent: XPIPE_BLOCKS per SM spread over the instances of the launch
-    int per = (XPIPE_BLOCKS * g_sms + nb - 1) / nb;
-    if (per > P.nrows) per = P.nrows;
-    if (per < 1) per = 1;
+    const int per = xpipe_blocks(P, nb);
     const size_t sm = 2 * XPIPE_BUF * sizeof(float2) + 128;   // + alignment slack
     if (P.nx == 1024) return launch_chain(k_xinv_pipe<REC, NM, true>, dim3(per, nb), dim3(XPASS_THREADS), sm, s, P, mat, Bf, A,
                                           map->map);

@@ -30,7 +30,14 @@ constexpr int XPASS_THREADS = 192;
 // holds 16 points of the x transform, 3 when it holds 32 (L = 512).
 constexpr int xpass_min_blocks(int L) { return (L >= 512 && !xpass_f3(L)) ? 3 : 5; }
 
-static inline int xthreads(const Plan& P) { return 3 * P.R * xpass_line_threads(P.L); }
+// Threads of an x-pass block of P.R rows: 192, or 96 when neither the
+// transform (3 R lines x N1 threads) nor the R nx cells ask for more.  Blocks
+// of few rows so have threads that hold no line: the cells of a row, not its
+// transform, are most of the work there.
+static inline int xthreads(const Plan& P) {
+    if (xpass_f3(P.L)) return XPASS_THREADS;
+    return 3 * P.R * xpass_line_threads(P.L) > 96 || P.R * P.nx > 96 ? XPASS_THREADS : 96;
+}
 
 // Rows per block: 64 lines of the transform per block, 3 R lines x N1 threads.
 __host__ __device__ constexpr int xpass_rows(int L) {

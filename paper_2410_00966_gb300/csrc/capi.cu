@@ -474,7 +474,7 @@ int mmcq_create(mmcq_t** out, const mmcq_grid* g, double Ms, double Aex, double 
     M.alpha = (float)alpha;
     M.vc = g->dx * g->dy * g->dz;
     M.hbar = h->hbar;
-    M.inv_hbar = 1.0 / h->hbar;
+    M.vc_hbar = M.vc / h->hbar;
 
     const long long BN = (long long)P.B * P.N;
     Buffers& Bf = h->Bf;
@@ -494,8 +494,8 @@ int mmcq_create(mmcq_t** out, const mmcq_grid* g, double Ms, double Aex, double 
     Bf.st = (InstState*)A(sizeof(InstState) * P.B);
     Bf.sc = (StageScalars*)A(sizeof(StageScalars) * P.B);
     // block partials: room for one row per block (the autotuner may lower P.R)
-    Bf.xpart = (double*)A(sizeof(double) * MAX_MODES * (long long)P.B * P.nrows);
-    Bf.mpart = (double*)A(sizeof(double) * 3LL * P.B * P.nrows);
+    Bf.xpart = (float4*)A(sizeof(float4) * MAX_MODES * (long long)P.B * P.nrows);
+    Bf.mpart = (float4*)A(sizeof(float4) * 3LL * P.B * P.nrows);
     Bf.mhist = nullptr;   // allocated by mmcq_set_recording
     Bf.epart = (float*)A(sizeof(float) * (long long)P.B * P.nrows);
     Bf.counter = (unsigned*)A(sizeof(unsigned) * P.B);

@@ -73,7 +73,7 @@ struct Material {
     float pre;        // -gamma / (1 + alpha^2)
     float alpha;
     double vc;        // cell volume
-    double hbar, inv_hbar;
+    double hbar, vc_hbar;   // vc_hbar = vc / hbar
 };
 
 // Per-instance parameters (set from the host).
@@ -135,12 +135,12 @@ struct Buffers {
     InstParams* ip;
     InstState* st;
     StageScalars* sc; // [B]
-    double* xpart;    // [MAX_MODES][B][x-pass blocks] FP64 partial coupling sums
+    float4* xpart;    // [MAX_MODES][B][x-pass blocks] partial coupling sums (Sum3)
     float* epart;     // [B][nrows] partial error maxima
     unsigned* counter;  // [B] blocks finished in the current kernel
     double* hist;     // [B][hcap] accepted step lengths
     int hcap;
-    double* mpart;    // [B][nrows-blocks][3] FP64 partial sums of m (recording only)
+    float4* mpart;    // [B][x-pass blocks][3] partial sums of m (Sum3; recording only)
     double* mhist;    // [B][hcap][4] t, <mx>, <my>, <mz> after accepted steps (recording only)
     int* flags;
     const float2* tw; // [twn] exp(-2 pi i k / twn)

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(
     const InstState& st = Bf.st[b];
     if (stage_skips(st, A)) return;
     if (blockIdx.x == 0) {
-        __shared__ double s_red[32 * (MAX_MODES + 3)];
+        __shared__ float4 s_red[32 * (MAX_MODES + 3)];
         __shared__ float s_redf[32];
         scalar_block(P, mat, Bf, A, b, s_red, s_redf);
         return;

@@ -1,6 +1,6 @@
 // Device code shared by the stage kernels (stage.cu, xinv.cu): Runge-Kutta
-// tableaux, the per-cell field / torque / RK update, the FP64 block
-// reductions and the per-instance scalar work.  Included by each translation
+// tableaux, the per-cell field / torque / RK update, the block
+// reductions and the per-instance FP64 scalar work.  Included by each translation
 // unit; constant-memory tables are per unit and filled by upload_tableaux().
 #pragma once
 
@@ -43,26 +43,65 @@ static __device__ double block_sum_d(double v, double* red) {
     return r;  // valid in thread 0
 }
 
-// Sums of the NQ doubles and the maximum of the float (with_max, uniform) of
+// A sum of FP32 terms kept as three floats: the rounding error of each addition
+// to h is computed exactly (Knuth's two-sum), that of the addition of those
+// errors to m likewise, and what is left goes to l.  72 bits against the 53 of
+// an FP64 accumulator, from FP32 additions only: this part issues two FP64
+// lanes per SM and clock, so that an FP64 add and conversion per cell took 32
+// of its clocks per warp against 3, and each of the ten dependent FP64 adds of
+// a block reduction about 300 clocks of latency against 100.
+struct Sum3 {
+    float h, m, l;
+};
+__device__ __forceinline__ float two_sum(float& a, float b) {   // a += b; the exact error
+    const float t = a + b, z = t - a, e = (a - (t - z)) + (b - z);
+    a = t;
+    return e;
+}
+__device__ __forceinline__ void sum3_add(Sum3& s, float x) {
+    const float e = two_sum(s.h, x);
+    s.l += two_sum(s.m, e);
+}
+__device__ __forceinline__ void sum3_merge(Sum3& s, const Sum3& o) {
+    const float e = two_sum(s.h, o.h), f = two_sum(s.m, o.m);
+    s.l = (s.l + o.l) + (f + two_sum(s.m, e));
+}
+__device__ __forceinline__ double sum3_value(const Sum3& s) { return (double)s.h + ((double)s.m + (double)s.l); }
+__device__ __forceinline__ Sum3 warp_sum3(Sum3 v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Sum3 w;
+        w.h = __shfl_down_sync(0xffffffffu, v.h, o);
+        w.m = __shfl_down_sync(0xffffffffu, v.m, o);
+        w.l = __shfl_down_sync(0xffffffffu, v.l, o);
+        sum3_merge(v, w);
+    }
+    return v;
+}
+__device__ __forceinline__ float4 sum3_pack(const Sum3& s) { return make_float4(s.h, s.m, s.l, 0.f); }
+__device__ __forceinline__ Sum3 sum3_unpack(const float4& f) { return Sum3{f.x, f.y, f.z}; }
+
+// Sums of the NQ terms and the maximum of the float (with_max, uniform) of
 // every thread, in one block barrier for all of them: the results are valid
 // in thread 0.  `red` holds NQ rows and `redf` one row of 32 warp values; the
-// caller synchronises before they are written again.
+// caller synchronises before they are written again.  Fixed order for a given
+// blockDim.
 template <int NQ>
-static __device__ __forceinline__ void block_reduce(double (&v)[NQ], float& mx, bool with_max, double* red,
+static __device__ __forceinline__ void block_reduce(Sum3 (&v)[NQ], float& mx, bool with_max, float4* red,
                                                     float* redf) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
 #pragma unroll
-    for (int q = 0; q < NQ; q++) v[q] = warp_sum_d(v[q]);
+    for (int q = 0; q < NQ; q++) v[q] = warp_sum3(v[q]);
     if (with_max) mx = warp_max_f(mx);
     if (l == 0) {
 #pragma unroll
-        for (int q = 0; q < NQ; q++) red[q * 32 + w] = v[q];
+        for (int q = 0; q < NQ; q++) red[q * 32 + w] = sum3_pack(v[q]);
         redf[w] = mx;
     }
     __syncthreads();
     if (w == 0) {
 #pragma unroll
-        for (int q = 0; q < NQ; q++) v[q] = warp_sum_d(l < nw ? red[q * 32 + l] : 0.0);
+        for (int q = 0; q < NQ; q++) v[q] = warp_sum3(l < nw ? sum3_unpack(red[q * 32 + l]) : Sum3{0.f, 0.f, 0.f});
         if (with_max) mx = warp_max_f(l < nw ? redf[l] : 0.f);
     }
 }
@@ -74,15 +113,6 @@ static __device__ double gamma_p(const InstParams& ip, const InstState& s, int k
     return e * cs * (ip.x0[k] - 2.0 * s.S[k] / hbar) - e * sn * (ip.p0[k] - 2.0 * s.C[k] / hbar);
 }
 
-// X / hbar from the product with the reciprocal and one correction step (the
-// division's own code is a long dependent chain on this part's FP64 pipe); the
-// division itself where that is not finite.
-__device__ __forceinline__ double over_hbar(double X, const Material& mat) {
-    const double q = X * mat.inv_hbar;
-    const double r = fma(fma(-q, mat.hbar, X), mat.inv_hbar, q);
-    return fabs(r) <= 1e300 ? r : X / mat.hbar;
-}
-
 // FP64 scalar work of one instance at the end of stage k, by one warp: lane
 // q < A.nmodes does mode q's arithmetic -- the amplitude (E-mode: d alpha_k/dt
 // = -(kappa_k + i omega_k) alpha_k + i X_k / hbar, Eq. eqmotionaclasical with
@@ -90,8 +120,8 @@ __device__ __forceinline__ double over_hbar(double X, const Material& mat) {
 // Cdiscrete) -- and lane 0 also time, accept / reject and step size.
 // load(): everything that does not depend on this stage's coupling sums: the
 // state (independent loads) and the Runge-Kutta sums over the earlier stages,
-// to run while the partials are on their way.  finish(): the rest, a few
-// dependent FP64 operations.  (One thread that copied the 750-byte state to its
+// to run while the partials are on their way.  finish(): the rest, as few
+// dependent FP64 operations as it takes (about 300 clocks each).  (One thread that copied the 750-byte state to its
 // stack and then did every mode took 4.7 us of a 20 us x inverse.)
 struct StageFinish {
     double dt, tcav;
@@ -148,7 +178,7 @@ struct StageFinish {
         const double X = Xsum * mat.vc;
         if (q < A.nmodes) s.X[q] = X;
         if (amp) {
-            di += over_hbar(X, mat);
+            di = fma(Xsum, mat.vc_hbar, di);
             s.ka_re[q][k] = dr;
             s.ka_im[q][k] = di;
             re += w * dr;
@@ -389,7 +419,7 @@ struct CellUpdate {
     // (Bx, By, Bz) holds demag + exchange on entry
     template <bool REC>
     __device__ __forceinline__ void run(const Material& mat, const Buffers& Bf, long long i, float4 m, float Bx,
-                                        float By, float Bz, double (&xacc)[NM], double (&macc)[REC ? 3 : 1],
+                                        float By, float Bz, Sum3 (&xacc)[NM], Sum3 (&macc)[REC ? 3 : 1],
                                         float& emax, bool& bad) const {
         const float Ms = m.w;
         float px_[NM], py_[NM], pz_[NM];
@@ -460,13 +490,12 @@ struct CellUpdate {
                 emax = fmaxf(emax, en);
             }
         }
-        // the coupling sums: each cell's product in FP32, promoted and
-        // accumulated in FP64 (thread, block and instance sums)
+        // the coupling sums: each cell's product in FP32, added without loss
 #pragma unroll
         for (int q = 0; q < NM; q++)
-            if (on[q]) xacc[q] += (double)(Ms * (mx.x * px_[q] + mx.y * py_[q] + mx.z * pz_[q]));
+            if (on[q]) sum3_add(xacc[q], Ms * (mx.x * px_[q] + mx.y * py_[q] + mx.z * pz_[q]));
         if constexpr (REC) {
-            if (Ms > 0.f) { macc[0] += mrec.x; macc[1] += mrec.y; macc[2] += mrec.z; }
+            if (Ms > 0.f) { sum3_add(macc[0], mrec.x); sum3_add(macc[1], mrec.y); sum3_add(macc[2], mrec.z); }
         }
     }
 };
@@ -495,50 +524,60 @@ __device__ __forceinline__ bool stage_records(const StageArgs& A, int k) {
 // other warps before the call.
 static __device__ __forceinline__ void finish_instance(const Plan& P, const Material& mat, const Buffers& Bf,
                                                        const StageArgs& A, int b, int k, StageFinish& f,
-                                                       double* s_red, float* s_redf,
+                                                       float4* s_red, float* s_redf,
                                                        const double (*trig)[MAX_MODES]) {
     const int n = A.nparts;
     const long long pb = (long long)b * n;
     const bool rec = stage_records(A, k), dp_last = A.kind == KIND_DP45 && k == 6;
     const InstParams& ip = Bf.ip[b];
     InstState& st = Bf.st[b];
-    double v[MAX_MODES + 3];
-#pragma unroll
-    for (int q = 0; q < MAX_MODES + 3; q++) v[q] = 0.0;
+    double msum[3] = {0.0, 0.0, 0.0}, x = 0.0;
     float em = 0.f;
     const long long ms = (long long)P.B * n;
+    const Sum3 z3 = {0.f, 0.f, 0.f};
     if (A.nmodes == 1 && !rec) {
-        double x[1] = {0.0};
+        Sum3 v[1] = {z3};
         for (int r = threadIdx.x; r < n; r += blockDim.x) {
-            x[0] += __ldcg(Bf.xpart + pb + r);
+            sum3_merge(v[0], sum3_unpack(__ldcg(Bf.xpart + pb + r)));
             if (dp_last) em = fmaxf(em, __ldcg(Bf.epart + pb + r));
         }
         if (threadIdx.x < 32) f.load(A, k, ip, st);
-        block_reduce<1>(x, em, dp_last, s_red, s_redf);
-        v[0] = x[0];
+        block_reduce<1>(v, em, dp_last, s_red, s_redf);
+        x = sum3_value(v[0]);
     } else {
+        Sum3 v[MAX_MODES + 3];
+#pragma unroll
+        for (int q = 0; q < MAX_MODES + 3; q++) v[q] = z3;
         for (int r = threadIdx.x; r < n; r += blockDim.x) {
 #pragma unroll
             for (int q = 0; q < MAX_MODES; q++)
-                if (q < A.nmodes) v[q] += __ldcg(Bf.xpart + q * ms + pb + r);
+                if (q < A.nmodes) sum3_merge(v[q], sum3_unpack(__ldcg(Bf.xpart + q * ms + pb + r)));
             if (dp_last) em = fmaxf(em, __ldcg(Bf.epart + pb + r));
             if (rec)
-                for (int c = 0; c < 3; c++) v[MAX_MODES + c] += __ldcg(Bf.mpart + 3 * (pb + r) + c);
+                for (int c = 0; c < 3; c++)
+                    sum3_merge(v[MAX_MODES + c], sum3_unpack(__ldcg(Bf.mpart + 3 * (pb + r) + c)));
         }
         if (threadIdx.x < 32) f.load(A, k, ip, st);
         block_reduce<MAX_MODES + 3>(v, em, dp_last, s_red, s_redf);
-    }
-    if (threadIdx.x < 32) {
-        double x = v[0];
-        if (A.nmodes > 1) {
+        if (threadIdx.x < 32) {
+            // lane q takes mode q's sum, lane 0 also the average's
+            if (rec)
+                for (int c = 0; c < 3; c++) msum[c] = sum3_value(v[MAX_MODES + c]);
+            Sum3 own = v[0];
 #pragma unroll
             for (int q = 0; q < MAX_MODES; q++) {
-                const double w = __shfl_sync(0xffffffffu, v[q], 0);
-                if (threadIdx.x == q) x = w;
+                Sum3 w;
+                w.h = __shfl_sync(0xffffffffu, v[q].h, 0);
+                w.m = __shfl_sync(0xffffffffu, v[q].m, 0);
+                w.l = __shfl_sync(0xffffffffu, v[q].l, 0);
+                if (threadIdx.x == q) own = w;
             }
+            x = sum3_value(own);
         }
+    }
+    if (threadIdx.x < 32) {
         em = __shfl_sync(0xffffffffu, em, 0);
-        f.finish(mat, A, k, ip, st, x, em, Bf.hist + (long long)b * Bf.hcap, Bf.hcap, Bf.flags, v + MAX_MODES,
+        f.finish(mat, A, k, ip, st, x, em, Bf.hist + (long long)b * Bf.hcap, Bf.hcap, Bf.flags, msum,
                  rec ? Bf.mhist + 4LL * b * Bf.hcap : nullptr, trig);
     }
 }
@@ -561,7 +600,7 @@ static __device__ __noinline__ void mode_trig(const InstParams& ip, int q, doubl
 // (P-mode: an exponential and a sine of each mode in every block, 9 us of a
 // 17 us x inverse of a 50^3 sphere with two modes).
 static __device__ __noinline__ void scalar_block(const Plan& P, const Material& mat, const Buffers& Bf,
-                                                 const StageArgs& A, int b, double* s_red, float* s_redf) {
+                                                 const StageArgs& A, int b, float4* s_red, float* s_redf) {
     __shared__ double s_end[3][MAX_MODES], s_now[3][MAX_MODES];
     const InstParams& ip = Bf.ip[b];
     const InstState& st = Bf.st[b];
@@ -589,18 +628,19 @@ static __device__ __noinline__ void scalar_block(const Plan& P, const Material& 
     __syncwarp();
     const int q = threadIdx.x;
     if (q < A.nmodes) {
-        double G = 0.0;
-        if (ip.cav_on[q])
-            G = A.mode == CAV_P ? gamma_p(ip, st, q, s_now[0][q], s_now[1][q], s_now[2][q], mat.hbar)
-                                : 2.0 * (A.field_only ? st.a_re[q] : (fin ? f.ar : st.as_re[q]));
-        Bf.sc[b].gamma[q] = (float)G;
+        float G = 0.f;
+        if (ip.cav_on[q]) {
+            if (A.mode == CAV_P) G = (float)gamma_p(ip, st, q, s_now[0][q], s_now[1][q], s_now[2][q], mat.hbar);
+            else G = 2.f * (float)(A.field_only ? st.a_re[q] : (fin ? f.ar : st.as_re[q]));
+        }
+        Bf.sc[b].gamma[q] = G;
     }
     if (q == MAX_MODES) Bf.sc[b].drive = (float)drive_factor(A, ip, st);
 }
 
 // The scalar work of this stage, by the last x inverse block to finish.
 static __device__ __noinline__ void finish_here(const Plan& P, const Material& mat, const Buffers& Bf,
-                                                const StageArgs& A, int b, double* s_red, float* s_redf) {
+                                                const StageArgs& A, int b, float4* s_red, float* s_redf) {
     __shared__ double s_end[3][MAX_MODES];
     if (threadIdx.x >= 32 && threadIdx.x < 32 + A.nmodes && A.mode == CAV_P && stage_last(A)) {
         const int q = threadIdx.x - 32;
@@ -618,9 +658,9 @@ static __device__ __noinline__ void finish_here(const Plan& P, const Material& m
 // next x forward does.  `part` = this block's index among A.nparts.
 template <bool REC, int NM>
 static __device__ __forceinline__ void stage_epilogue(const Plan& P, const Material& mat, const Buffers& Bf,
-                                                      const StageArgs& A, int b, int part, const double (&xacc)[NM],
-                                                      float emax, bool bad, double* s_red, float* s_redf, int* s_last,
-                                                      const double* macc) {
+                                                      const StageArgs& A, int b, int part, const Sum3 (&xacc)[NM],
+                                                      float emax, bool bad, float4* s_red, float* s_redf, int* s_last,
+                                                      const Sum3* macc) {
     // RK4: a non-finite torque is an error.  DP45: it marks the attempt, which
     // is then rejected with the smallest step factor (an overflowing trial
     // step); a state that stays non-finite ends in step-size underflow.
@@ -631,7 +671,7 @@ static __device__ __forceinline__ void stage_epilogue(const Plan& P, const Mater
     const int nparts = A.nparts;
     const bool dp_last = A.kind == KIND_DP45 && A.stage == 6;
     constexpr int NQ = NM + (REC ? 3 : 0);
-    double v[NQ];
+    Sum3 v[NQ];
 #pragma unroll
     for (int q = 0; q < NM; q++) v[q] = xacc[q];
     if constexpr (REC)
@@ -642,10 +682,10 @@ static __device__ __forceinline__ void stage_epilogue(const Plan& P, const Mater
         const int nm = NM == 1 ? 1 : A.nmodes;
 #pragma unroll
         for (int q = 0; q < NM; q++)
-            if (q < nm) Bf.xpart[((long long)q * P.B + b) * nparts + part] = v[q];
+            if (q < nm) Bf.xpart[((long long)q * P.B + b) * nparts + part] = sum3_pack(v[q]);
         if (dp_last) Bf.epart[pb + part] = emax;
         if constexpr (REC)
-            for (int c = 0; c < 3; c++) Bf.mpart[3 * (pb + part) + c] = v[NM + c];
+            for (int c = 0; c < 3; c++) Bf.mpart[3 * (pb + part) + c] = sum3_pack(v[NM + c]);
         if (A.fin_here) {
             __threadfence();
             unsigned prev = atomicAdd(Bf.counter + b, 1u);

@@ -4,7 +4,7 @@
 // excitation) + cavity sum_k B_rms,k Gamma_k (Sec. 2.1 field terms, Eq. bcav),
 // the LLG torque (Eq. llg), the RK bookkeeping, and block partials of the
 // coupling sums X_k = V_c sum_i Ms_i m_i . B_rms,k,i (Eq. gammafinal): each
-// cell's FP32 product promoted and added in FP64.  The partials are reduced in
+// cell's FP32 product added in three floats (Sum3).  The partials are reduced in
 // a fixed order, and the cavity amplitudes and the step-size controller
 // advanced in FP64, by the scalar block of the next x forward or, at the end
 // of an attempt or of a call, by the instance's last block to finish.
@@ -50,7 +50,7 @@ template <int NM, bool REC>
 __device__ __forceinline__ void xinv_cells(const Plan& P, const Material& mat, const Buffers& Bf,
                                            const CellUpdate<NM>& cu, const float2* xs, int ld, const float4* msrc,
                                            long long base, int nx, int nr, int nthr, const int2* s_yz,
-                                           double (&xacc)[NM], double (&macc)[REC ? 3 : 1], float& emax, bool& bad) {
+                                           Sum3 (&xacc)[NM], Sum3 (&macc)[REC ? 3 : 1], float& emax, bool& bad) {
     const bool want_demag = cu.want_demag, want_exch = cu.want_exch;
     const int pl = nx * P.ny;
     // cell ii = r nx + x of the block; (x, r) advance by the block size
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(
     constexpr int NPT = F3 ? 16 : ColShape<L>::NPT, N1 = xpass_line_threads(L);
     constexpr int RF = xpass_rows(L);
     extern __shared__ float2 sm[];
-    __shared__ double s_red[32 * (MAX_MODES + 3)];
+    __shared__ float4 s_red[32 * (MAX_MODES + 3)];
     __shared__ float s_redf[32];
     __shared__ int s_last;
     __shared__ int2 s_yz[64];                          // rows per block <= 64
@@ -247,10 +247,10 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(
 
     CellUpdate<NM> cu;
     cu.init(Bf, A, st, ip, Bf.sc[b], cb, (long long)A.inst0 * P.N);
-    double xacc[NM];
+    Sum3 xacc[NM];
 #pragma unroll
-    for (int q = 0; q < NM; q++) xacc[q] = 0.0;
-    double macc[REC ? 3 : 1] = {};
+    for (int q = 0; q < NM; q++) xacc[q] = Sum3{0.f, 0.f, 0.f};
+    Sum3 macc[REC ? 3 : 1] = {};
     float emax = 0.f;
     bool bad = false;
     xinv_cells<NM, REC>(P, mat, Bf, cu, xs, ld, msrc, base, nx, nr, nthr, s_yz, xacc, macc, emax, bad);
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(
     extern __shared__ __align__(128) float2 sm_raw[];  // [2][XPIPE_BUF] from the first 128-byte boundary
     float2* sm = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(sm_raw) + 127) & ~(uintptr_t)127);
     __shared__ __align__(8) unsigned long long s_bar[2];
-    __shared__ double s_red[32 * (MAX_MODES + 3)];
+    __shared__ float4 s_red[32 * (MAX_MODES + 3)];
     __shared__ float s_redf[32];
     __shared__ int s_last;
     __shared__ int2 s_yz[1];
@@ -329,10 +329,10 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(
 
     CellUpdate<NM> cu;
     cu.init(Bf, A, st, ip, Bf.sc[b], cb, (long long)A.inst0 * P.N);
-    double xacc[NM];
+    Sum3 xacc[NM];
 #pragma unroll
-    for (int q = 0; q < NM; q++) xacc[q] = 0.0;
-    double macc[REC ? 3 : 1] = {};
+    for (int q = 0; q < NM; q++) xacc[q] = Sum3{0.f, 0.f, 0.f};
+    Sum3 macc[REC ? 3 : 1] = {};
     float emax = 0.f;
     bool bad = false;
     const int line = threadIdx.x / N1, j = threadIdx.x % N1;

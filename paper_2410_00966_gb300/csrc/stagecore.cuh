@@ -181,8 +181,12 @@ struct StageFinish {
             di = fma(Xsum, mat.vc_hbar, di);
             s.ka_re[q][k] = dr;
             s.ka_im[q][k] = di;
-            re += w * dr;
-            im += w * di;
+            // (not at DP45's last stage: a rejected attempt may have overflowed,
+            // and alpha_q must stay what it was)
+            if (!(last && K == KIND_DP45)) {
+                re += w * dr;
+                im += w * di;
+            }
         }
         if (!last) {
             if (amp) {

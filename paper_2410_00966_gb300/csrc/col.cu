@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(512) k_col_reg(Plan Pl, Buffers Bf, StageArgs 
     const int b = A.inst0 + blockIdx.z;
     const int c0 = ncomp == 3 ? 0 : blockIdx.x % 3;
     const int bx = ncomp == 3 ? blockIdx.x : blockIdx.x / 3;
+    chain_wait();
     if (stage_skips(Bf.st[b], A)) return;
     const int TX = FIXED ? WC / 3 : Pl.TX;
     const int lt = FIXED ? ilog2<(FIXED ? WC / 3 : 1)>() : Pl.lt;
@@ -159,6 +160,7 @@ template <int P>
 __global__ void __launch_bounds__(256) k_zconv(Plan Pl, Buffers Bf, StageArgs A, ColArgs C) {
     extern __shared__ float2 sm[];      // [P][W]
     const int b = A.inst0 + blockIdx.z;
+    chain_wait();
     if (stage_skips(Bf.st[b], A)) return;
     const int TX = Pl.TX, lt = Pl.lt;
     const int W = C.G * 3 * TX;
@@ -305,6 +307,7 @@ __global__ void __launch_bounds__(192, 6) k_zconv2(Plan Pl, Buffers Bf, StageArg
     extern __shared__ float2 sm[];      // [P][W]
     constexpr bool FIXED = TXC > 0 && GC > 0;
     const int b = A.inst0 + blockIdx.z;
+    chain_wait();
     if (stage_skips(Bf.st[b], A)) return;
     const int TX = FIXED ? TXC : Pl.TX, lt = FIXED ? ilog2<(TXC > 0 ? TXC : 1)>() : Pl.lt;
     const int Gb = FIXED ? GC : C.G;
@@ -444,6 +447,7 @@ __global__ void __launch_bounds__(512, (FIXED && PH == 1024) ? 2 : 1) k_col_spli
     const int c0 = ncomp == 3 ? 0 : bxx % 3;
     const int bx = ncomp == 3 ? bxx : bxx / 3;
     // the same for both blocks of a cluster (same instance)
+    chain_wait();
     if (stage_skips(Bf.st[b], A)) return;
     const int TX = FIXED ? 8 : Pl.TX, lt = FIXED ? 3 : Pl.lt;
     const int G = FIXED ? 1 : C.G;
@@ -577,6 +581,7 @@ __global__ void __launch_bounds__(MAX_THREADS) k_col_gen(Plan P, Buffers Bf, Sta
     const int b = A.inst0 + blockIdx.z;
     const int c0 = C.ncomp == 3 ? 0 : blockIdx.x % 3;
     const int bx = C.ncomp == 3 ? blockIdx.x : blockIdx.x / 3;
+    chain_wait();
     if (stage_skips(Bf.st[b], A)) return;
     const int TX = P.TX;
     const int rw = C.ncomp * TX;

@@ -6,7 +6,9 @@
 namespace mq {
 
 // Host side: launch a stage-chain kernel; cluster > 1 groups consecutive
-// blocks along x into clusters of that size.
+// blocks along x into clusters of that size.  Programmatic dependent launch:
+// the blocks are placed as the last blocks of the kernel before end, and
+// chain_wait() holds each of them until that kernel's writes are visible.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_chain_cl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                                    int cluster, Args... args) {
@@ -15,13 +17,15 @@ inline cudaError_t launch_chain_cl(void (*kernel)(KArgs...), dim3 grid, dim3 blo
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cluster;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 template <typename... KArgs, typename... Args>
@@ -29,6 +33,16 @@ inline cudaError_t launch_chain(void (*kernel)(KArgs...), dim3 grid, dim3 block,
                                 Args... args) {
     return launch_chain_cl(kernel, grid, block, smem, s, 1, args...);
 }
+
+// Every stage-chain kernel calls this before it reads or writes anything that
+// another kernel writes or reads: wait for the kernel before.  The kernels do
+// not ask for the next one early (griddepcontrol.launch_dependents): its
+// blocks would take room from this one's and from other streams' kernels
+// (largest grid 13.0 against 11.7 ms per 2 attempts, the batched map 29.2
+// against 27.4 ms).  Placing them as this one's last blocks end is enough:
+// 32x32 film 5.09 -> 3.78 ms per 50 steps, 300x120x5 strip 1.32 -> 1.13 ms per
+// 3 attempts, largest grid 11.82 -> 11.72 ms.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 // Whether this instance does nothing in this launch.
 __device__ __forceinline__ bool stage_skips(const InstState& s, const StageArgs& A) {

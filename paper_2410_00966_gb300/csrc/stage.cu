@@ -39,6 +39,26 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(
     constexpr int RF = xpass_rows(L);
     extern __shared__ float2 sm[];
     const int b = A.inst0 + blockIdx.y;
+    const int Rb = FX ? RF : P.R;
+    const int nx = FX ? L : P.nx;
+    const int px = FX ? 2 * L : P.px;
+    const int nthr = FX ? 3 * RF * N1 : (int)blockDim.x;
+    const int ld = xpass_ld(Rb);
+    float2* zs = sm;
+    // exp(-2 pi i e / px), e < px: a shared copy for the four-step transform;
+    // the three-factor one (L = 1024) reads the global table through L1
+    float2* stw = sm + xpass_fft_rows(L) * ld;
+    const int tws = P.twn / px;
+    if (blockIdx.x != 0) {
+        if constexpr (!F3)
+            for (int e = threadIdx.x; e < px; e += nthr) stw[e] = __ldg(Bf.tw + e * tws);
+        // rows nx/2.. of the packed line are zero padding (rows below are all
+        // written).  FX (nx = L): they are not stored, the transform takes its
+        // points n2 >= NPT / 2 as zeros.
+        if constexpr (!FX)
+            for (int i = (nx >> 1) * ld + threadIdx.x; i < L * ld; i += nthr) zs[i] = make_float2(0.f, 0.f);
+    }
+    chain_wait();
     const InstState& st = Bf.st[b];
     if (stage_skips(st, A)) return;
     if (blockIdx.x == 0) {
@@ -47,38 +67,20 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(
         scalar_block(P, mat, Bf, A, b, s_red, s_redf);
         return;
     }
-    const int Rb = FX ? RF : P.R;
-    const int nx = FX ? L : P.nx;
-    const int px = FX ? 2 * L : P.px;
-    const int nthr = FX ? 3 * RF * N1 : (int)blockDim.x;
     const int row0 = ((int)blockIdx.x - 1) * Rb;
     const int nr = FX ? RF : min(P.R, P.nrows - row0);
-    const int ld = xpass_ld(Rb);
     const long long base = (long long)b * P.N + (long long)row0 * nx;
     const float4* m0 = Bf.m[st.mcur] + base;
     StageInput si;
     si.init(Bf, A, st, base);
     if (threadIdx.x == 0) {
         // the block's rows of m0 and of every k it combines: in flight while
-        // the shared tables are set up
+        // the block synchronises
         const unsigned bytes = (unsigned)(nr * nx * sizeof(float4));
         prefetch_l2(m0, bytes);
         si.prefetch(Bf, bytes);
     }
-    float2* zs = sm;
-    // exp(-2 pi i e / px), e < px: a shared copy for the four-step transform;
-    // the three-factor one (L = 1024) reads the global table through L1
-    float2* stw = sm + xpass_fft_rows(L) * ld;
-    const int tws = P.twn / px;
-    if constexpr (!F3)
-        for (int e = threadIdx.x; e < px; e += nthr) stw[e] = __ldg(Bf.tw + e * tws);
-    // rows nx/2.. of the packed line are zero padding (rows below are all
-    // written).  FX (nx = L): they are not stored, the transform takes its
-    // points n2 >= NPT / 2 as zeros.
-    if constexpr (!FX)
-        for (int i = (nx >> 1) * ld + threadIdx.x; i < L * ld; i += nthr) zs[i] = make_float2(0.f, 0.f);
     __syncthreads();
-
 
     for (int i = threadIdx.x; i < nr * nx; i += nthr) {
         float4 v = m0[i];

@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(
     __shared__ int s_last;
     __shared__ int2 s_yz[64];                          // rows per block <= 64
     const int b = A.inst0 + blockIdx.y;
+    chain_wait();
     const InstState& st = Bf.st[b];
     if (stage_skips(st, A)) return;
     const InstParams& ip = Bf.ip[b];
@@ -291,6 +292,7 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(
     __shared__ int s_last;
     __shared__ int2 s_yz[1];
     const int b = A.inst0 + blockIdx.y;
+    chain_wait();
     const InstState& st = Bf.st[b];
     if (stage_skips(st, A)) return;
     const InstParams& ip = Bf.ip[b];

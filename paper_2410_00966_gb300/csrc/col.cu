@@ -14,6 +14,7 @@
 //   between the forward and the inverse z transform.
 // k_col_split<PH, FIXED>: y passes whose padded length 2 PH exceeds the
 //   register path, as two PH-point register transforms per column.
+// k_conv_2048: the 2-D convolution of 513 to 1024 rows of cells.
 // k_col_gen: any power-of-two length, shared-memory Stockham (fft.cuh); the
 //   remaining long transforms.
 #include <algorithm>
@@ -574,6 +575,162 @@ __global__ void __launch_bounds__(512, (FIXED && PH == 1024) ? 2 : 1) k_col_spli
     }
 }
 
+// 2-D convolution for py = 2048 (513 to 1024 rows of cells): y transform,
+// product and inverse of one 2-column tile (6 columns of 2048 points) per
+// block.  The radix-4 Stockham stages of block_fft, same operations in the same
+// order, but two stages at a time in registers (16 points per thread, 128
+// threads per column), so that each direction goes through shared memory three
+// times instead of six; the first pass reads global memory (rows of padding are
+// zeros in registers) and the last writes it.  Bound by instruction issue and
+// shared memory (104 KB, one block of 24 warps per SM).  1000x600 film:
+// 176 us (k_col_gen) -> 64 us per field evaluation.
+//
+// Passes 1 and 2 (stages Ns, 4 Ns with Ns = 1, 16): thread t takes rows
+// t + 128 m; v[r' + 4 r''] is input r'' of butterfly t + 128 r' of the first
+// stage, and v[r + 4 s] ends as row base + (s + 4 r) Ns.
+constexpr int CONV2K_T = 128, CONV2K_W = 6;
+__device__ __forceinline__ int conv2k_at(int row) { return (row + (row >> 4)) * CONV2K_W; }   // padded against bank conflicts
+constexpr size_t CONV2K_SMEM = (size_t)(2048 + 128) * CONV2K_W * sizeof(float2);
+
+template <int NS, bool INV>
+__device__ __forceinline__ void conv2k_pass16(float2 (&v)[16], int t, const float2* __restrict__ tw, int twn) {
+    const int jm = t & (NS - 1);
+    float2 a[4];
+    auto mul = [&](float2 x, int k) {
+        const float2 w = __ldg(tw + k);
+        return INV ? cmulc(x, w) : cmul(x, w);
+    };
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+#pragma unroll
+        for (int r = 0; r < 4; r++) a[r] = v[q + 4 * r];
+        if (NS > 1) {
+#pragma unroll
+            for (int r = 1; r < 4; r++) a[r] = mul(a[r], jm * r * (twn / (4 * NS)));
+        }
+        radix4(a, INV);
+#pragma unroll
+        for (int r = 0; r < 4; r++) v[q + 4 * r] = a[r];
+    }
+#pragma unroll
+    for (int s = 0; s < 4; s++) {
+        const int jb = jm + s * NS;
+#pragma unroll
+        for (int r = 0; r < 4; r++) a[r] = r == 0 ? v[4 * s] : mul(v[r + 4 * s], jb * r * (twn / (16 * NS)));
+        radix4(a, INV);
+#pragma unroll
+        for (int r = 0; r < 4; r++) v[r + 4 * s] = a[r];
+    }
+}
+template <int NS>
+__device__ __forceinline__ void conv2k_store16(const float2 (&v)[16], float2* sm, int t, int col) {
+    const int base = (t / NS) * (16 * NS) + (t & (NS - 1));
+#pragma unroll
+    for (int s = 0; s < 4; s++)
+#pragma unroll
+        for (int r = 0; r < 4; r++) sm[conv2k_at(base + (s + 4 * r) * NS) + col] = v[r + 4 * s];
+}
+__device__ __forceinline__ void conv2k_load16(float2 (&v)[16], const float2* sm, int t, int col) {
+#pragma unroll
+    for (int m = 0; m < 16; m++) v[m] = sm[conv2k_at(t + CONV2K_T * m) + col];
+}
+// Pass 3 (stages 256 and 1024): v[8 h + r' + 2 r] holds row jm + 256 r' + 512 r
+// with jm = t + 128 h; on exit v[8 h + 2 r + u] is row jm + 256 r + 1024 u.
+__device__ __forceinline__ void conv2k_load8(float2 (&v)[16], const float2* sm, int t, int col) {
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+#pragma unroll
+            for (int r = 0; r < 4; r++) v[8 * h + q + 2 * r] = sm[conv2k_at(t + 128 * h + 256 * q + 512 * r) + col];
+}
+template <bool INV>
+__device__ __forceinline__ void conv2k_pass8(float2 (&v)[16], int t, const float2* __restrict__ tw, int twn) {
+    auto mul = [&](float2 x, int k) {
+        const float2 w = __ldg(tw + k);
+        return INV ? cmulc(x, w) : cmul(x, w);
+    };
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int jm = t + 128 * h;
+        float2 a[2][4];
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+#pragma unroll
+            for (int r = 0; r < 4; r++)
+                a[q][r] = r == 0 ? v[8 * h + q] : mul(v[8 * h + q + 2 * r], jm * r * (twn / 1024));
+            radix4(a[q], INV);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            const float2 w = mul(a[1][r], (jm + 256 * r) * (twn / 2048));
+            v[8 * h + 2 * r] = cadd(a[0][r], w);
+            v[8 * h + 2 * r + 1] = csub(a[0][r], w);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(CONV2K_T * CONV2K_W, 1) k_conv_2048(Plan P, Buffers Bf, StageArgs A, ColArgs C) {
+    extern __shared__ float2 sm[];      // [2048 + 128][6]
+    const int b = A.inst0 + blockIdx.z;
+    chain_wait();
+    if (stage_skips(Bf.st[b], A)) return;
+    const int col = threadIdx.x % CONV2K_W, t = threadIdx.x / CONV2K_W;
+    const float2* in = C.in + b * C.in_b + blockIdx.x * C.in_t + col;
+    float2* out = C.out + b * C.out_b + blockIdx.x * C.out_t + col;
+    float2 v[16];
+#pragma unroll
+    for (int m = 0; m < 16; m++) {
+        const int r = t + CONV2K_T * m;
+        v[m] = m < 8 && r < C.n_in ? in[r * CONV2K_W] : make_float2(0.f, 0.f);
+    }
+    conv2k_pass16<1, false>(v, t, Bf.tw, P.twn);
+    conv2k_store16<1>(v, sm, t, col);
+    __syncthreads();
+    conv2k_load16(v, sm, t, col);
+    conv2k_pass16<16, false>(v, t, Bf.tw, P.twn);
+    __syncthreads();
+    conv2k_store16<16>(v, sm, t, col);
+    __syncthreads();
+    conv2k_load8(v, sm, t, col);
+    conv2k_pass8<false>(v, t, Bf.tw, P.twn);
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+            sm[conv2k_at(t + 128 * h + 256 * (q >> 1) + 1024 * (q & 1)) + col] = v[8 * h + q];
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * 2048; i += CONV2K_T * CONV2K_W) {
+        const int r = i >> 1, tx = i & 1;
+        float2* p = sm + conv2k_at(r) + tx;
+        float2 mx = p[0], my = p[2], mz = p[4];
+        demag_product(P, Bf.kern, blockIdx.x * 2 + tx, r, 0, mx, my, mz);
+        p[0] = mx; p[2] = my; p[4] = mz;
+    }
+    __syncthreads();
+    conv2k_load16(v, sm, t, col);
+    conv2k_pass16<1, true>(v, t, Bf.tw, P.twn);
+    __syncthreads();
+    conv2k_store16<1>(v, sm, t, col);
+    __syncthreads();
+    conv2k_load16(v, sm, t, col);
+    conv2k_pass16<16, true>(v, t, Bf.tw, P.twn);
+    __syncthreads();
+    conv2k_store16<16>(v, sm, t, col);
+    __syncthreads();
+    conv2k_load8(v, sm, t, col);
+    conv2k_pass8<true>(v, t, Bf.tw, P.twn);
+    // rows below 1024 (u = 0) are the ones kept
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+            const int row = t + 128 * h + 256 * r;
+            if (row < C.n_out) out[row * CONV2K_W] = v[8 * h + 2 * r];
+        }
+}
+
 // Generic shared-memory version (any power-of-two P up to 4096).
 template <int SLOTS>
 __global__ void __launch_bounds__(MAX_THREADS) k_col_gen(Plan P, Buffers Bf, StageArgs A, ColArgs C) {
@@ -799,6 +956,9 @@ cudaError_t launch_conv_part(const Plan& P, const Buffers& Bf, const StageArgs& 
         C.fwd = 1; C.mult = 1; C.inv = 1; C.ncomp = 3; C.ky_is_row = 1;
         C.group_tiles = 1; C.nouter = 1;
         C.G = tuned_groups(T, 0, pick_groups(3 * P.TX, P.py, P.NT, COL_MAX_THREADS, COL_SMEM_CAP));
+        // (tiles are 2 columns wide at this length, see col_fits)
+        if (P.py == 2048 && P.TX == 2 && P.ny <= 1024)
+            return launch_chain(k_conv_2048, dim3(P.NT, 1, nb), dim3(CONV2K_T * CONV2K_W), CONV2K_SMEM, s, P, Bf, A, C);
     } else if (part == 1 || part == 3) {
         bool fwd = part == 1;
         C.in = fwd ? Bf.spec : Bf.spec2;
@@ -921,6 +1081,7 @@ cudaError_t col_init() {
     const int lim = 200 * 1024;
     if ((e = cudaFuncSetAttribute(k_col_gen<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_col_gen<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_conv_2048, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) return e;
 #define MMCQ_SET(Pv, Wv)                                                                                 \
     if ((e = cudaFuncSetAttribute(k_col_reg<Pv, Wv>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != \
         cudaSuccess)                                                                                        \

@@ -85,28 +85,30 @@ __device__ __forceinline__ void block_product(const Plan& P, const Buffers& Bf, 
 // column.  Groups are consecutive kx tiles (y passes) or consecutive outer
 // indices (z pass); in both cases consecutive columns are adjacent in memory.
 // Transform lengths with a fixed-shape instantiation of k_col_reg.
-constexpr bool col_fixed_len(int P) { return P >= 64 && P <= 512; }
+// (three components in 48 KB of shared memory: 256 at most)
+constexpr bool col_fixed_len(int P) { return P >= 64 && P <= 256; }
 
 // WC > 0: the block is one kx tile of WC / 3 columns with all three
 // components (G = 1), rows WC apart in both spectra, fixed at compile time so
 // that the row and shared-memory offsets are immediates.
-template <int P, int WC>
-__global__ void __launch_bounds__(512) k_col_reg(Plan Pl, Buffers Bf, StageArgs A, ColArgs C) {
+// NC (with WC > 0): components per block, 3 or 1.
+template <int P, int WC, int NC = 3>
+__device__ __forceinline__ void col_reg_body(const Plan& Pl, const Buffers& Bf, const StageArgs& A, const ColArgs& C) {
     constexpr int NPT = ColShape<P>::NPT, N1 = ColShape<P>::N1;
     constexpr bool FIXED = WC > 0;
     extern __shared__ float2 sm[];
-    const int ncomp = FIXED ? 3 : C.ncomp;
+    const int ncomp = FIXED ? NC : C.ncomp;
     const int b = A.inst0 + blockIdx.z;
     const int c0 = ncomp == 3 ? 0 : blockIdx.x % 3;
     const int bx = ncomp == 3 ? blockIdx.x : blockIdx.x / 3;
     chain_wait();
     if (stage_skips(Bf.st[b], A)) return;
-    const int TX = FIXED ? WC / 3 : Pl.TX;
-    const int lt = FIXED ? ilog2<(FIXED ? WC / 3 : 1)>() : Pl.lt;
+    const int TX = FIXED ? WC / NC : Pl.TX;
+    const int lt = FIXED ? ilog2<(FIXED ? WC / NC : 1)>() : Pl.lt;
     const int G = FIXED ? 1 : C.G;
     const int rw = ncomp * TX;
     const int W = G * rw;
-    const long long in_r = FIXED ? WC : C.in_r, out_r = FIXED ? WC : C.out_r;
+    const long long in_r = FIXED ? 3 * (WC / NC) : C.in_r, out_r = FIXED ? 3 * (WC / NC) : C.out_r;
     const int col = threadIdx.x % W;
     const int j = threadIdx.x / W;
     const int g = ncomp == 3 ? (col >> lt) / 3 : (col >> lt);
@@ -126,7 +128,7 @@ __global__ void __launch_bounds__(512) k_col_reg(Plan Pl, Buffers Bf, StageArgs 
         v[n2] = (valid && r < C.n_in) ? in[r * in_r] : make_float2(0.f, 0.f);
     }
     if (C.fwd) col_fft<P, false>(v, sm, W, col, j, Bf.tw, Pl.twn);
-    if (C.mult) {
+    if (!FIXED && C.mult) {
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < NPT; i++) sm[col_out_row<P>(j, i) * W + col] = v[i];
@@ -144,6 +146,21 @@ __global__ void __launch_bounds__(512) k_col_reg(Plan Pl, Buffers Bf, StageArgs 
         const int r = transformed ? col_out_row<P>(j, i) : j + N1 * i;
         if (r < C.n_out) out[r * out_r] = v[i];
     }
+}
+
+template <int P, int WC>
+__global__ void __launch_bounds__(512) k_col_reg(Plan Pl, Buffers Bf, StageArgs A, ColArgs C) {
+    col_reg_body<P, WC>(Pl, Bf, A, C);
+}
+
+// The y passes of 512 and 1024 points: one component of one 8-column tile per
+// block at compile time, 32 points per thread (96 registers and 5 blocks per
+// SM at 512 points; the generic shape took 128 and spilled).  16 x 256x256x4
+// grids: y forward 77 -> 67 us.
+template <int P>
+__global__ void __launch_bounds__(8 * ColShape<P>::N1, P == 512 ? 5 : 2)
+    k_col_reg1(Plan Pl, Buffers Bf, StageArgs A, ColArgs C) {
+    col_reg_body<P, 8, 1>(Pl, Bf, A, C);
 }
 
 // z pass of the 3-D convolution for pz <= 32, one thread per (component, ky,
@@ -797,6 +814,11 @@ static cudaError_t launch_reg(const Plan& Pl, const Buffers& Bf, const StageArgs
             return launch_chain(k_col_reg<P, 24>, grid, W * N1, (size_t)P * W * sizeof(float2), s, Pl, Bf, A, C);
         }
     }
+    if constexpr (P == 512 || P == 1024) {
+        // the y passes of these lengths run one component per block
+        if (Pl.TX == 8 && C.ncomp == 1 && C.G == 1 && !C.mult && C.group_tiles && C.in_r == 24 && C.out_r == 24)
+            return launch_chain(k_col_reg1<P>, grid, W * N1, (size_t)P * W * sizeof(float2), s, Pl, Bf, A, C);
+    }
     (void)fixed;
     return launch_chain(k_col_reg<P, 0>, grid, W * N1, (size_t)P * W * sizeof(float2), s, Pl, Bf, A, C);
 }
@@ -1088,7 +1110,13 @@ cudaError_t col_init() {
         return e;
     MMCQ_SET(1, 0) MMCQ_SET(2, 0) MMCQ_SET(4, 0) MMCQ_SET(8, 0) MMCQ_SET(16, 0) MMCQ_SET(32, 0) MMCQ_SET(64, 0)
     MMCQ_SET(128, 0) MMCQ_SET(256, 0) MMCQ_SET(512, 0) MMCQ_SET(1024, 0)
-    MMCQ_SET(64, 24) MMCQ_SET(128, 24) MMCQ_SET(256, 24) MMCQ_SET(512, 24)
+    MMCQ_SET(64, 24) MMCQ_SET(128, 24) MMCQ_SET(256, 24)
+#undef MMCQ_SET
+#define MMCQ_SET(Pv)                                                                                       \
+    if ((e = cudaFuncSetAttribute(k_col_reg1<Pv>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != \
+        cudaSuccess)                                                                                         \
+        return e;
+    MMCQ_SET(512) MMCQ_SET(1024)
 #undef MMCQ_SET
 #define MMCQ_SET(Pv)                                                                                            \
     if ((e = cudaFuncSetAttribute(k_zconv<Pv>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) \

@@ -420,8 +420,10 @@ struct CellUpdate {
                              : (s < 6 ? Bf.k[s == 0 ? k1slot : s] : Bf.k[k1slot == 0 ? 6 : 0]);
     }
 
-    // (Bx, By, Bz) holds demag + exchange on entry
-    template <bool REC>
+    // (Bx, By, Bz) holds demag + exchange on entry.  MID: a stage that stores
+    // its torque and is not the last of its step, with every field term on
+    // (all but one launch of a step): none of the checks below is made per cell
+    template <bool REC, bool MID>
     __device__ __forceinline__ void run(const Material& mat, const Buffers& Bf, long long i, float4 m, float Bx,
                                         float By, float Bz, Sum3 (&xacc)[NM], Sum3 (&macc)[REC ? 3 : 1],
                                         float& emax, bool& bad) const {
@@ -430,12 +432,12 @@ struct CellUpdate {
 #pragma unroll
         for (int q = 0; q < NM; q++) px_[q] = py_[q] = pz_[q] = 0.f;
         if (Ms > 0.f) {
-            if (want_anis) {
+            if ((MID || want_anis) && mat.two_ku != 0.f) {
                 float mu = m.x * mat.u[0] + m.y * mat.u[1] + m.z * mat.u[2];
                 float f = mat.two_ku * __fdividef(mu, Ms);
                 Bx += f * mat.u[0]; By += f * mat.u[1]; Bz += f * mat.u[2];
             }
-            if (want_zee) { Bx += bex; By += bey; Bz += bez; }
+            if (MID || want_zee) { Bx += bex; By += bey; Bz += bez; }
 #pragma unroll
             for (int q = 0; q < NM; q++) {
                 // the excitation (Appendix C) uses the map of mode 0
@@ -446,11 +448,11 @@ struct CellUpdate {
                 } else {
                     py_[q] = bs[q];
                 }
-                if (on[q] && want_cav) { Bx += G[q] * px_[q]; By += G[q] * py_[q]; Bz += G[q] * pz_[q]; }
-                if (q == 0 && want_zee) { Bx += D * px_[0]; By += D * py_[0]; Bz += D * pz_[0]; }
+                if (on[q] && (MID || want_cav)) { Bx += G[q] * px_[q]; By += G[q] * py_[q]; Bz += G[q] * pz_[q]; }
+                if (q == 0 && (MID || want_zee)) { Bx += D * px_[0]; By += D * py_[0]; Bz += D * pz_[0]; }
             }
         }
-        if (field_only) {
+        if (!MID && field_only) {
             Bf.fout[i - fb] = make_float4(Bx, By, Bz, 0.f);
             return;
         }
@@ -464,7 +466,9 @@ struct CellUpdate {
         if (!(fabsf(kk.x + kk.y + kk.z) <= 3.0e38f)) bad = true;
         float4 mx = m;   // m used for the coupling sums of this launch
         float4 mrec = m; // state being accepted (recorded spatial average)
-        if (K == KIND_RK4) {
+        if (MID) {
+            kout[i] = kk;
+        } else if (K == KIND_RK4) {
             if (s < 3) {
                 kout[i] = kk;
             } else {

@@ -46,12 +46,12 @@ __device__ __forceinline__ int zfast_row(const Plan& P, int i) {
     return (i - y * P.nz) * P.ny + y;
 }
 
-template <int NM, bool REC>
+template <int NM, bool REC, bool MID>
 __device__ __forceinline__ void xinv_cells(const Plan& P, const Material& mat, const Buffers& Bf,
                                            const CellUpdate<NM>& cu, const float2* xs, int ld, const float4* msrc,
                                            long long base, int nx, int nr, int nthr, const int2* s_yz,
                                            Sum3 (&xacc)[NM], Sum3 (&macc)[REC ? 3 : 1], float& emax, bool& bad) {
-    const bool want_demag = cu.want_demag, want_exch = cu.want_exch;
+    const bool want_demag = MID || cu.want_demag, want_exch = MID || cu.want_exch;
     const int pl = nx * P.ny;
     // cell ii = r nx + x of the block; (x, r) advance by the block size
     const int stepr = nthr / nx, stepx = nthr - stepr * nx;
@@ -94,7 +94,7 @@ __device__ __forceinline__ void xinv_cells(const Plan& P, const Material& mat, c
             const float inv = Ms > 0.f ? __fdividef(1.f, Ms) : 0.f;
             Bx += hxy.x * inv; By += hxy.y * inv; Bz += hz * inv;
         }
-        cu.template run<REC>(mat, Bf, i, m, Bx, By, Bz, xacc, macc, emax, bad);
+        cu.template run<REC, MID>(mat, Bf, i, m, Bx, By, Bz, xacc, macc, emax, bad);
         x += stepx;
         r += stepr;
         if (x >= nx) { x -= nx; r++; }
@@ -111,7 +111,8 @@ __device__ __forceinline__ void xinv_cells(const Plan& P, const Material& mat, c
 // instantiations so that the common launches carry no extra accumulators.
 // FX: the fixed shape of the large grids (rows of nx = L cells, XPASS_ROWS(L)
 // rows per block with none left over, tiles of 8 kx columns) at compile time.
-template <int L, bool REC, int NM, bool FX>
+// MID: a middle stage (see CellUpdate::run), for the fixed shape.
+template <int L, bool REC, int NM, bool FX, bool MID = false>
 __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(
     const __grid_constant__ Plan P, const __grid_constant__ Material mat, const __grid_constant__ Buffers Bf,
     const __grid_constant__ StageArgs A) {
@@ -254,8 +255,8 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xinv(
     Sum3 macc[REC ? 3 : 1] = {};
     float emax = 0.f;
     bool bad = false;
-    xinv_cells<NM, REC>(P, mat, Bf, cu, xs, ld, msrc, base, nx, nr, nthr, s_yz, xacc, macc, emax, bad);
-    if (A.field_only) return;
+    xinv_cells<NM, REC, MID>(P, mat, Bf, cu, xs, ld, msrc, base, nx, nr, nthr, s_yz, xacc, macc, emax, bad);
+    if (!MID && A.field_only) return;
     stage_epilogue<REC, NM>(P, mat, Bf, A, b, blockIdx.x, xacc, emax, bad, s_red, s_redf, &s_last, macc);
 }
 
@@ -279,7 +280,7 @@ static int g_sms = 0;                                        // SMs of the devic
 
 __device__ __forceinline__ int xpipe_land(int k, int c) { return 24 * (k >> 3) + 8 * c + (k & 7); }
 
-template <bool REC, int NM, bool FX>
+template <bool REC, int NM, bool FX, bool MID = false>
 __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(
     const __grid_constant__ Plan P, const __grid_constant__ Material mat, const __grid_constant__ Buffers Bf,
     const __grid_constant__ StageArgs A, const __grid_constant__ TensorMap tm) {
@@ -381,11 +382,11 @@ __global__ void __launch_bounds__(XPASS_THREADS, XPIPE_BLOCKS) k_xinv_pipe(
             for (int i = 0; i < NPT; i++) xs[col3_out_row<L>(j, i) * ld + line] = v[i];
         }
         __syncthreads();
-        xinv_cells<NM, REC>(P, mat, Bf, cu, xs, ld, msrc, cb + (long long)row * nx, nx, 1, nthr, s_yz, xacc, macc,
+        xinv_cells<NM, REC, MID>(P, mat, Bf, cu, xs, ld, msrc, cb + (long long)row * nx, nx, 1, nthr, s_yz, xacc, macc,
                             emax, bad);
         __syncthreads();   // buffer q and s_yz are rewritten by the next rows
     }
-    if (A.field_only) return;
+    if (!MID && A.field_only) return;
     stage_epilogue<REC, NM>(P, mat, Bf, A, b, blockIdx.x, xacc, emax, bad, s_red, s_redf, &s_last, macc);
 }
 
@@ -406,11 +407,20 @@ int xinv_parts(const Plan& P, const Buffers& Bf, int nb, const SpecMap* map, con
     return xpipe_applies(P, Bf, map) && (!T || T->x_pipe != 0) ? xpipe_blocks(P, nb) : P.nblk;
 }
 
+// A middle stage with every field term on (CellUpdate::run).
+static bool stage_mid(const StageArgs& A) {
+    return !A.field_only && A.terms == 31 && A.stage < (A.kind == KIND_RK4 ? 3 : 6);
+}
+
 template <bool REC, int NM>
 static cudaError_t launch_xpipe(const Plan& P, const Material& mat, const Buffers& Bf, const StageArgs& A, int nb,
                          const SpecMap* map, cudaStream_t s) {
     const int per = xpipe_blocks(P, nb);
     const size_t sm = 2 * XPIPE_BUF * sizeof(float2) + 128;   // + alignment slack
+    if constexpr (!REC && NM == 1)
+        if (P.nx == 1024 && stage_mid(A))
+            return launch_chain(k_xinv_pipe<false, 1, true, true>, dim3(per, nb), dim3(XPASS_THREADS), sm, s, P, mat, Bf, A,
+                                map->map);
     if (P.nx == 1024) return launch_chain(k_xinv_pipe<REC, NM, true>, dim3(per, nb), dim3(XPASS_THREADS), sm, s, P, mat, Bf, A,
                                           map->map);
     return launch_chain(k_xinv_pipe<REC, NM, false>, dim3(per, nb), dim3(XPASS_THREADS), sm, s, P, mat, Bf, A, map->map);
@@ -433,8 +443,10 @@ cudaError_t launch_xinv(const Plan& P, const Material& mat, const Buffers& Bf, c
     }
     if (!multi && !rec && xpass_fixed(P)) {
         switch (P.L) {
-#define MMCQ_CASE(Lv) \
-    case Lv: return launch_chain(k_xinv<Lv, false, 1, true>, grid, th, sm, s, P, mat, Bf, A);
+#define MMCQ_CASE(Lv)                                                                                          \
+    case Lv:                                                                                                   \
+        if (stage_mid(A)) return launch_chain(k_xinv<Lv, false, 1, true, true>, grid, th, sm, s, P, mat, Bf, A); \
+        return launch_chain(k_xinv<Lv, false, 1, true>, grid, th, sm, s, P, mat, Bf, A);
             MMCQ_XFIXED(MMCQ_CASE)
 #undef MMCQ_CASE
             default: break;
@@ -473,8 +485,9 @@ cudaError_t xinv_init() {
     if ((e = xinv_attr(k_xinv<Lv, true, MAX_MODES, false>, lim)) != cudaSuccess) return e;
     MMCQ_XCASES(MMCQ_CASE)
 #undef MMCQ_CASE
-#define MMCQ_CASE(Lv) \
-    if ((e = xinv_attr(k_xinv<Lv, false, 1, true>, lim)) != cudaSuccess) return e;
+#define MMCQ_CASE(Lv)                                                              \
+    if ((e = xinv_attr(k_xinv<Lv, false, 1, true>, lim)) != cudaSuccess) return e; \
+    if ((e = xinv_attr(k_xinv<Lv, false, 1, true, true>, lim)) != cudaSuccess) return e;
     MMCQ_XFIXED(MMCQ_CASE)
 #undef MMCQ_CASE
 #define MMCQ_PIPE(R, M)                                                                 \
@@ -482,6 +495,7 @@ cudaError_t xinv_init() {
     if ((e = xinv_attr(k_xinv_pipe<R, M, false>, lim)) != cudaSuccess) return e;
     MMCQ_PIPE(false, 1) MMCQ_PIPE(true, 1) MMCQ_PIPE(false, MAX_MODES) MMCQ_PIPE(true, MAX_MODES)
 #undef MMCQ_PIPE
+    if ((e = xinv_attr(k_xinv_pipe<false, 1, true, true>, lim)) != cudaSuccess) return e;
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;

@@ -137,6 +137,38 @@ __global__ void __launch_bounds__(XPASS_THREADS, xpass_min_blocks(L)) k_xfwd(
     // tile t of a row holds the 3 TX values (c, tx) contiguously; when 3 TX
     // divides the block, a thread keeps one (c, tx) and steps over the tiles
     const int w3 = 3 * TX;
+    if constexpr (FX) {
+        // X[k] and X[L-k] together: with E and w D of k, those of L - k are
+        // conj E and (w D.x, -w D.y) (the table's W^{L-k} is -conj W^k), so a
+        // pair takes the reads, the twiddle and the product of one value, bit
+        // for bit (x forward of 16 x 256x256x4 71 -> 64 us).  The padding
+        // columns beyond L are zero from the start and never written.
+        const int e = threadIdx.x % 24, t0 = threadIdx.x / 24;
+        const int c = e >> 3, tx = e & 7;
+        constexpr int DT = 3 * RF * N1 / 24;
+        for (int r = 0; r < RF; r++) {
+            const int row = row0 + r;
+            const int z = (int)fdiv((unsigned)row, P.fd_ny), y = row - z * P.ny;
+            float2* out = Bf.spec + (((long long)b * P.nz + z) * NT * P.ny + y) * 24 + 8 * c;
+            const int line = 3 * r + c;
+#pragma unroll 2
+            for (int k = 8 * t0 + tx; k <= L / 2; k += 8 * DT) {
+                const int kc = L - k;
+                const float2 Zk = zs[k * ld + line], Zc = conjf2(zs[(k == 0 ? 0 : kc) * ld + line]);
+                const float2 E = make_float2(0.5f * (Zk.x + Zc.x), 0.5f * (Zk.y + Zc.y));
+                const float2 D = make_float2(0.5f * (Zk.x - Zc.x), 0.5f * (Zk.y - Zc.y));
+                const float2 wD = cmul(F3 ? __ldg(Bf.tw + k * tws) : stw[k], D);
+                out[(k >> 3) * tstride + (k & 7)] = make_float2(__fadd_rn(E.x, wD.y), __fsub_rn(E.y, wD.x));
+                if (k == 0) {       // X[L], by its own formula (E and D of k = L are those of k = 0)
+                    const float2 wL = cmul(F3 ? __ldg(Bf.tw + L * tws) : stw[L], D);
+                    out[(L >> 3) * tstride] = make_float2(__fadd_rn(E.x, wL.y), __fsub_rn(E.y, wL.x));
+                } else if (k != L / 2) {
+                    out[(kc >> 3) * tstride + (kc & 7)] = make_float2(__fsub_rn(E.x, wD.y), __fsub_rn(-E.y, wD.x));
+                }
+            }
+        }
+        return;
+    }
     if (nthr % w3 == 0) {
         const int e = threadIdx.x % w3, t0 = threadIdx.x / w3, dtt = nthr / w3;
         const int c = e >> lt, tx = e & (TX - 1);

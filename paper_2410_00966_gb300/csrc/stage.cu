@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(CSUM_THREADS) k_coupling_part(const float4* m0
                                                                 const InstState* st, const float4* prof, long long N,
                                                                 int b0, double* part, int nblk) {
     __shared__ double red[32];
+    chain_wait();
     const int b = b0 + blockIdx.y;
     const float4* m = (st[b].mcur ? m1 : m0) + (long long)b * N;
     const long long chunk = (N + nblk - 1) / nblk;
@@ -273,6 +274,7 @@ __global__ void __launch_bounds__(CSUM_THREADS) k_coupling_part(const float4* m0
 __global__ void __launch_bounds__(CSUM_THREADS) k_coupling_fin(const InstParams* ip, const double* part, int nblk,
                                                                double vc, int b0, int k, double* out) {
     __shared__ double red[32];
+    chain_wait();
     const int b = b0 + blockIdx.x;
     double acc = 0.0;
     for (int q = threadIdx.x; q < nblk; q += CSUM_THREADS) acc += part[(long long)blockIdx.x * nblk + q];
@@ -418,10 +420,10 @@ cudaError_t launch_get_field(const float4* f, float* dst, long long N, cudaStrea
 }
 cudaError_t launch_coupling_sum(const Buffers& Bf, long long N, double vc, int b0, int nb, int k, double* out,
                                 cudaStream_t s) {
-    k_coupling_part<<<dim3(Bf.cpart_n, nb), CSUM_THREADS, 0, s>>>(Bf.m[0], Bf.m[1], Bf.st, Bf.prof[k], N, b0,
-                                                                  Bf.cpart, Bf.cpart_n);
-    k_coupling_fin<<<nb, CSUM_THREADS, 0, s>>>(Bf.ip, Bf.cpart, Bf.cpart_n, vc, b0, k, out);
-    return cudaGetLastError();
+    const cudaError_t e = launch_chain(k_coupling_part, dim3(Bf.cpart_n, nb), dim3(CSUM_THREADS), 0, s, Bf.m[0], Bf.m[1], Bf.st,
+                                       Bf.prof[k], N, b0, Bf.cpart, Bf.cpart_n);
+    if (e != cudaSuccess) return e;
+    return launch_chain(k_coupling_fin, dim3(nb), dim3(CSUM_THREADS), 0, s, Bf.ip, Bf.cpart, Bf.cpart_n, vc, b0, k, out);
 }
 cudaError_t launch_set_dt(InstState* st, int B, double dt, cudaStream_t s) {
     k_set_dt<<<(B + 127) / 128, 128, 0, s>>>(st, B, dt);

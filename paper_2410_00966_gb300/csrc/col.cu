@@ -8,7 +8,8 @@
 // k_col_reg<P, WC>: transform length P <= 1024 in registers (fftreg.cuh);
 //   a thread group owns one column and loads its strided rows straight from
 //   global memory (consecutive threads = consecutive columns = contiguous
-//   memory).  WC > 0: the common tile shape fixed at compile time.
+//   memory).  WC > 0: the common tile shape fixed at compile time; k_col_reg1
+//   the same for one component per block (512 and 1024 points).
 // k_zconv<P> / k_zconv2<P, TXC, GC>: the z pass (pz <= 32, one thread per
 //   column / pz = 16 or 32, two threads per column) with the demag product
 //   between the forward and the inverse z transform.

@@ -92,7 +92,7 @@ struct InstParams {
 struct InstState {
     double t, tcav, dt, t_end;
     double a_re[MAX_MODES], a_im[MAX_MODES];     // alpha_k at the start of the step (E-mode)
-    double as_re[MAX_MODES], as_im[MAX_MODES];   // alpha_k of the stage about to be evaluated (E-mode)
+    double as_re[MAX_MODES], as_im[MAX_MODES];   // alpha_k of the last stage prepared after the first (E-mode)
     double S[MAX_MODES], C[MAX_MODES];           // P-mode accumulators
     double ka_re[MAX_MODES][MAX_STAGES], ka_im[MAX_MODES][MAX_STAGES];
     double X[MAX_MODES];    // last reduced coupling sums (include V_c)

@@ -118,7 +118,7 @@ struct mmcq {
     int rows_rule = 1;      // most x-pass rows per block of the fixed rule
     int x_rows = 1;         // the same of the current plan
     int sms = 0;            // SMs of the device
-    int64_t tune_epoch = 0; // bumped when the launch parameters change (groups capture again)
+    int64_t epoch = 0;      // bumped when the launch parameters or a buffer of Bf change (groups capture again)
 };
 
 enum { CLS_XFWD = 0, CLS_CONV2D, CLS_YFWD, CLS_ZCONV, CLS_YINV, CLS_XINV, NCLS };
@@ -663,6 +663,7 @@ int mmcq_set_cavity_mode(mmcq_t* h, int inst, int mode, double omega_c, double k
         if (!h->Bf.prof[mode]) {
             h->Bf.prof[mode] = (float4*)dev_alloc(h, sizeof(float4) * N);
             if (!h->Bf.prof[mode]) return fail(h, MMCQ_ERR_CUDA, "profile allocation failed");
+            h->epoch++;
         }
         std::vector<float4> p(N);
         for (long long i = 0; i < N; i++) p[i] = make_float4(profile[3 * i], profile[3 * i + 1], profile[3 * i + 2], 0.f);
@@ -966,6 +967,7 @@ int mmcq_set_recording(mmcq_t* h, int every) {
     if (every > 0 && !h->Bf.mhist) {
         h->Bf.mhist = (double*)dev_alloc(h, sizeof(double) * 4LL * h->P.B * h->Bf.hcap);
         if (!h->Bf.mhist) return fail(h, MMCQ_ERR_CUDA, "device allocation failed");
+        h->epoch++;
     }
     h->record = every;
     return MMCQ_OK;
@@ -1055,7 +1057,7 @@ bool tune_apply(mmcq_t* h, const mmcq_tuning* t) {
         h->tune.x_pipe = t->x_pipe;
         set_rows(h, t->x_rows);
     }
-    h->tune_epoch++;
+    h->epoch++;
     return true;
 }
 
@@ -1612,7 +1614,7 @@ struct mmcq_group {
     std::vector<cudaEvent_t> join, in;
     cudaGraphExec_t exec = nullptr;
     std::vector<int> cap_kind, cap_mode, cap_record, cap_nmodes;
-    std::vector<int64_t> cap_epoch;         // tuning epoch of each handle at the capture
+    std::vector<int64_t> cap_epoch;         // epoch of each handle at the capture
     std::vector<double> cap_tol;
     std::vector<int64_t> cap_launches;      // kernel launches per replay, per handle
     int64_t replays = 0;
@@ -1638,7 +1640,7 @@ bool group_stale(const mmcq_group_t* g) {
     for (size_t i = 0; i < g->hs.size(); i++) {
         const mmcq_t* h = g->hs[i];
         if (h->kind != g->cap_kind[i] || h->mode != g->cap_mode[i] || h->tol != g->cap_tol[i] ||
-            h->record != g->cap_record[i] || h->nmodes != g->cap_nmodes[i] || h->tune_epoch != g->cap_epoch[i])
+            h->record != g->cap_record[i] || h->nmodes != g->cap_nmodes[i] || h->epoch != g->cap_epoch[i])
             return true;
     }
     return false;
@@ -1678,7 +1680,7 @@ int group_capture(mmcq_group_t* g) {
         g->cap_tol[i] = g->hs[i]->tol;
         g->cap_record[i] = g->hs[i]->record;
         g->cap_nmodes[i] = g->hs[i]->nmodes;
-        g->cap_epoch[i] = g->hs[i]->tune_epoch;
+        g->cap_epoch[i] = g->hs[i]->epoch;
     }
     if (r != MMCQ_OK) {
         if (graph) cudaGraphDestroy(graph);

@@ -959,7 +959,10 @@ int mmcq_set_drive(mmcq_t* h, int inst, double amp, double omega_cut, double t0)
             h->ip[b].drv_wcut = omega_cut;
             h->ip[b].drv_t0 = t0;
         }
-    return upload_params(h);
+    int r = upload_params(h);
+    if (r) return r;
+    // the excitation is part of every stage's field: a kept first stage is stale
+    return edit_state(h, inst, [](InstState& s, int) { s.have_k1 = 0; });
 }
 
 int mmcq_set_recording(mmcq_t* h, int every) {

@@ -124,3 +124,17 @@ def test_step_clipped_by_a_new_horizon_with_a_kept_first_stage():
         r.sim.set_horizon(0.0)
         r.step(2)
     r.check("horizon")
+
+
+def test_first_stage_after_a_changed_drive_sees_the_new_drive():
+    """The excitation acts in every stage: its change drops the kept first
+    stage.  (20 mT over a step of a few ps turns m by some 1e-4 in the first
+    stage's share of it.)"""
+    require_gpu()
+    r = _Run()
+    amp = 0.02 / np.abs(r.o.get_brms()).max()
+    r.step(6, 1e-12)
+    for i in range(6):
+        r.both(lambda h: h.set_drive((amp, -0.5 * amp, 0.0)[i % 3], 2 * math.pi * 1e10, r.sim.cavity()["t"]))
+        r.step(2)
+    r.check("drive")

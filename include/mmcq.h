@@ -384,14 +384,13 @@ const char* mmcq_group_last_error(const mmcq_group_t* g);
  *                  in a block of its own (the inverse's two blocks a cluster
  *                  exchanging terms through shared memory), 0 both halves in
  *                  one block; -1: no choice.
- * mmcq_autotune times one middle Runge-Kutta stage of the whole batch (stage
- *   input, transforms, field, torque, coupling sums, per-instance finish) at
- *   the current state under the fixed rules and under each candidate, one knob
- *   at a time with the others at their best so far, with events around every
- *   pass: a candidate is kept when the passes its knob changes (both x passes
- *   for x_rows, the column part for col_groups, the z pass for z_split, the x
- *   inverse for x_pipe, the y pass for y_split) take less time, by the median of `reps` stages.  The
- *   fastest plan stays in use for the later steps of the handle.  Only that stage's scratch buffers are written and the
+ * mmcq_autotune times a middle Runge-Kutta stage of the whole batch as a step
+ *   launches it (stage input, transforms, field, torque, coupling sums,
+ *   per-instance finish; a few stages in a row) at the current state under the
+ *   fixed rules and under each candidate, one knob at a time with the others at
+ *   their best so far: a candidate is kept when its stage takes less time, by
+ *   the median of `reps` runs.  The fastest plan stays in use for the later
+ *   steps of the handle.  Only that stage's scratch buffers are written and the
  *   instance states are restored, so the integration is unchanged.  The choice
  *   is also cached for the process (per device, grid and batch size): a later
  *   handle of the same shape gets it without timing (out->candidates = 0).
@@ -406,9 +405,9 @@ typedef struct {
     int z_split;
     int x_pipe;
     int y_split[2];
-    double eval_ms;        /* one stage of the batch with this plan: sum of the passes' median times */
+    double eval_ms;        /* median time of one stage of the batch with this plan */
     double rule_ms;        /* the same with the fixed rules */
-    int candidates;        /* plans timed (0: taken from the cache) */
+    int candidates;        /* plans tried (0: taken from the cache) */
 } mmcq_tuning;
 int mmcq_autotune(mmcq_t* h, int reps, mmcq_tuning* out);
 int mmcq_set_tuning(mmcq_t* h, const mmcq_tuning* t);

@@ -1098,97 +1098,90 @@ int mmcq_autotune(mmcq_t* h, int reps, mmcq_tuning* out) {
     if (r) return r;
     const Plan& P = h->P;
     const int B = P.B;
-    // timed: one middle Runge-Kutta stage of the whole batch (stage input,
-    // transforms, field, torque, coupling sums and the per-instance finish),
-    // which writes only that stage's scratch buffers and the instance states;
-    // the states are put back afterwards, so the integration is unchanged
+    // timed: a middle Runge-Kutta stage of the whole batch as a step launches
+    // it (stage input, transforms, field, torque, coupling sums, the scalar
+    // work of the stage before beside the x forward), several in a row with
+    // nothing between their kernels.  It writes only that stage's scratch
+    // buffers and the instance states; the states are put back afterwards, so
+    // the integration is unchanged.  (Events between the passes would keep
+    // each kernel from being placed as the one before ends, and judge a knob on
+    // launches that no step makes: 40x40 film 33 us a stage, steps 16 us.)
     std::vector<InstState> saved(B);
     CK(h, cudaStreamSynchronize(h->stream));
     CK(h, cudaMemcpy(saved.data(), h->Bf.st, sizeof(InstState) * B, cudaMemcpyDeviceToHost));
     StageArgs A = step_args(h);
     A.stage = h->kind == KIND_RK4 ? 1 : 3;
     A.record = 0;
-    // passes of one stage: 0 = x forward, 1..4 = column parts 0..3, 5 = x inverse;
-    // events bracket each pass so that a knob is judged on the passes it changes
+    A.fin_here = 0;
     const int parts0 = P.nz == 1 ? 0 : 1, parts1 = P.nz == 1 ? 0 : 3;
-    std::vector<cudaEvent_t> ev;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
     int err = MMCQ_OK;
     auto cleanup = [&]() -> int {
-        for (auto e : ev) cudaEventDestroy(e);
+        for (auto e : ev) if (e) cudaEventDestroy(e);
         if (cudaStreamSynchronize(h->stream) != cudaSuccess ||
             cudaMemcpy(h->Bf.st, saved.data(), sizeof(InstState) * B, cudaMemcpyHostToDevice) != cudaSuccess)
             return MMCQ_ERR_CUDA;
         return MMCQ_OK;
     };
-    const int nev = 2 + (parts1 - parts0 + 1) + 1;    // start, after x forward, after each part, after x inverse
-    for (int q = 0; q < nev; q++) {
-        cudaEvent_t e = nullptr;
+    for (auto& e : ev)
         if (cudaEventCreate(&e) != cudaSuccess) {
             cleanup();
             return fail(h, MMCQ_ERR_CUDA, "autotune: event creation failed");
         }
-        ev.push_back(e);
-    }
     int ncand = 0;
-    auto eval = [&](bool timed) -> cudaError_t {
+    // first: the stage before has left no partials of this plan to finish
+    auto eval = [&](bool first) -> cudaError_t {
         cudaError_t e;
-        int q = 0;
         A.nparts = xinv_parts(h->P, h->Bf, B, &h->spec_map, &h->tune);
-        if (timed && (e = cudaEventRecord(ev[q++], h->stream)) != cudaSuccess) return e;
+        A.fin_prev = first ? -1 : A.stage - 1;
         if ((e = launch_xfwd(h->P, h->mat, h->Bf, A, B, h->stream)) != cudaSuccess) return e;
-        if (timed && (e = cudaEventRecord(ev[q++], h->stream)) != cudaSuccess) return e;
-        for (int part = parts0; part <= parts1; part++) {
+        for (int part = parts0; part <= parts1; part++)
             if ((e = launch_conv_part(h->P, h->Bf, A, B, h->stream, part, &h->tune)) != cudaSuccess) return e;
-            if (timed && (e = cudaEventRecord(ev[q++], h->stream)) != cudaSuccess) return e;
-        }
-        if ((e = launch_xinv(h->P, h->mat, h->Bf, A, B, h->stream, &h->spec_map, &h->tune)) != cudaSuccess) return e;
-        if (timed && (e = cudaEventRecord(ev[q++], h->stream)) != cudaSuccess) return e;
-        return cudaSuccess;
+        return launch_xinv(h->P, h->mat, h->Bf, A, B, h->stream, &h->spec_map, &h->tune);
     };
-    // median time per pass over `reps` stages, after one untimed; pass k is
-    // slot 0 (x forward), 1 + part, or 5 (x inverse)
-    auto measure = [&](double (&ms)[6]) -> int {
-        std::vector<std::vector<float>> t(6, std::vector<float>(reps, 0.f));
-        if (eval(false) != cudaSuccess) return MMCQ_ERR_CUDA;
-        for (int q = 0; q < reps; q++) {
-            if (eval(true) != cudaSuccess || cudaEventSynchronize(ev[nev - 1]) != cudaSuccess) return MMCQ_ERR_CUDA;
-            std::vector<int> slot;
-            slot.push_back(0);
-            for (int part = parts0; part <= parts1; part++) slot.push_back(1 + part);
-            slot.push_back(5);
-            for (size_t k = 0; k < slot.size(); k++)
-                if (cudaEventElapsedTime(&t[slot[k]][q], ev[k], ev[k + 1]) != cudaSuccess) return MMCQ_ERR_CUDA;
+    // median time of a stage over `reps` chains of `chain`, after one untimed
+    // stage and one untimed chain
+    const int chain = 4;
+    auto measure = [&](double& ms) -> int {
+        std::vector<float> t(reps, 0.f);
+        if (eval(true) != cudaSuccess) return MMCQ_ERR_CUDA;
+        for (int q = -1; q < reps; q++) {
+            if (cudaEventRecord(ev[0], h->stream) != cudaSuccess) return MMCQ_ERR_CUDA;
+            for (int k = 0; k < chain; k++)
+                if (eval(false) != cudaSuccess) return MMCQ_ERR_CUDA;
+            if (cudaEventRecord(ev[1], h->stream) != cudaSuccess || cudaEventSynchronize(ev[1]) != cudaSuccess ||
+                cudaEventElapsedTime(&t[q < 0 ? 0 : q], ev[0], ev[1]) != cudaSuccess)
+                return MMCQ_ERR_CUDA;
         }
-        for (int k = 0; k < 6; k++) {
-            std::sort(t[k].begin(), t[k].end());
-            ms[k] = t[k][reps / 2];
-        }
-        ncand++;
+        std::sort(t.begin(), t.end());
+        ms = t[reps / 2] / chain;
         return MMCQ_OK;
     };
-    auto total = [](const double (&ms)[6]) { return ms[0] + ms[1] + ms[2] + ms[3] + ms[4] + ms[5]; };
     mmcq_tuning best{};
     tune_apply(h, nullptr);
     tune_read(h, &best);
-    double rule[6], cur[6];
-    if ((err = measure(rule))) {
+    double rule_ms = 0.0, best_ms = 0.0;
+    ncand++;
+    if ((err = measure(rule_ms))) {
         cleanup();
         return fail(h, err, "autotune: timing failed");
     }
-    std::copy(rule, rule + 6, cur);
-    // one knob at a time, the others at their best so far, judged on the
-    // passes that knob changes (slots)
-    auto trial = [&](const mmcq_tuning& c, std::initializer_list<int> slots) -> int {
+    best_ms = rule_ms;
+    // one knob at a time, the others at their best so far
+    auto trial = [&](const mmcq_tuning& c) -> int {
         mmcq_tuning t = c;
+        const int R = h->P.R;
         if (!tune_apply(h, &t)) return MMCQ_OK;
-        double ms[6];
-        int e = measure(ms);
-        if (e) return e;
-        double a = 0, b = 0;
-        for (int k : slots) { a += ms[k]; b += cur[k]; }
-        if (a < b) {
-            best = t;
-            for (int k : slots) cur[k] = ms[k];
+        ncand++;
+        // (rows that the rule had chosen already: the launches of the plan in use)
+        if (t.x_rows == best.x_rows || h->P.R != R) {
+            double ms;
+            int e = measure(ms);
+            if (e) return e;
+            if (ms < best_ms) {
+                best = t;
+                best_ms = ms;
+            }
         }
         tune_apply(h, &best);
         return MMCQ_OK;
@@ -1196,33 +1189,32 @@ int mmcq_autotune(mmcq_t* h, int reps, mmcq_tuning* out) {
     for (int R = h->rows_rule / 2; R >= 1 && R >= h->rows_rule / 4 && !err; R /= 2) {
         mmcq_tuning c = best;
         c.x_rows = R;
-        err = trial(c, {0, 5});
+        err = trial(c);
     }
     int gmax[4], zc, zr, yc, yr[2];
     conv_tunables(P, gmax, &zc, &zr, &yc, yr);
     if (zc && !err) {
         mmcq_tuning c = best;
         c.z_split = 1 - zr;
-        err = trial(c, {3});
+        err = trial(c);
     }
     for (int k = 0; k < 2 && yc && !err; k++) {
         mmcq_tuning c = best;
         c.y_split[k] = 1 - yr[k];
-        err = trial(c, {k == 0 ? 2 : 4});
+        err = trial(c);
     }
     for (int k = 0; k < 4 && !err; k++) {
         for (int G = 1; G < gmax[k] && !err; G *= 2) {
             mmcq_tuning c = best;
             c.col_groups[k] = G;
-            err = trial(c, {1 + k});
+            err = trial(c);
         }
     }
     if (h->spec_map.valid && !err) {
         mmcq_tuning c = best;
         c.x_pipe = 0;
-        err = trial(c, {5});
+        err = trial(c);
     }
-    const double rule_ms = total(rule), best_ms = total(cur);
     if (cleanup() != MMCQ_OK) err = MMCQ_ERR_CUDA;
     if (err) {
         tune_apply(h, nullptr);

@@ -367,9 +367,10 @@ const char* mmcq_group_last_error(const mmcq_group_t* g);
  * The paper runs Mumax3's fixed kernels; here the launch shape of each pass of
  * the field evaluation is chosen per grid by timing.  The knobs change no data
  * layout and no arithmetic, so every plan computes the same field:
- *   x_rows         most cell rows per block of the x passes (1 .. the rule's
- *                  count; a grid that so few blocks leave the GPU idle on takes
- *                  fewer rows per block);
+ *   x_rows         cell rows per block of the x passes, 1 up to the largest
+ *                  count of the grid's row length; that largest count, which a
+ *                  handle starts with, stands for the rule: as many, or as few
+ *                  as keep two blocks on every SM;
  *   col_groups[k]  kx tiles (y passes) or ky columns (z pass) per block of the
  *                  column passes: k = 0 the 2-D convolution, 1 the forward y,
  *                  2 the z pass, 3 the inverse y (0: not launched for this

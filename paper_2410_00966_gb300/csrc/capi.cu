@@ -115,8 +115,8 @@ struct mmcq {
     int post_head = 0, post_count = 0;
     SpecMap spec_map{};     // TMA map of the x-half-spectrum (pipelined x inverse)
     Tune tune{{0, 0, 0, 0}, -1, -1, {-1, -1}};   // launch parameters chosen by mmcq_autotune (default: the fixed rules)
-    int rows_rule = 1;      // most x-pass rows per block of the fixed rule
-    int x_rows = 1;         // the same of the current plan
+    int rows_rule = 1;      // most x-pass rows per block
+    int x_rows = 1;         // rows of the current plan (rows_rule: the rule's choice up to that)
     int sms = 0;            // SMs of the device
     int64_t epoch = 0;      // bumped when the launch parameters or a buffer of Bf change (groups capture again)
 };
@@ -195,11 +195,12 @@ int upload_params(mmcq_t* h) {
     return MMCQ_OK;
 }
 
-// At most `most` rows per x-pass block (fewer on a grid that would otherwise
-// leave the GPU idle).
-void set_rows(mmcq_t* h, int most) {
-    h->x_rows = most;
-    h->P.R = rows_within(most, (long long)h->P.nrows * h->P.B, h->sms);
+// Rows per x-pass block of a plan: rows_rule, the most there can be, leaves the
+// number to the rule (fewer on a grid that would otherwise leave the GPU idle);
+// a smaller number is taken as it is.
+void set_rows(mmcq_t* h, int rows) {
+    h->x_rows = rows;
+    h->P.R = rows < h->rows_rule ? rows : rows_within(rows, (long long)h->P.nrows * h->P.B, h->sms);
     h->P.nblk = (h->P.nrows + h->P.R - 1) / h->P.R;
 }
 

@@ -43,28 +43,38 @@ static __device__ double block_sum_d(double v, double* red) {
     return r;  // valid in thread 0
 }
 
-// A sum of FP32 terms kept as three floats: the rounding error of each addition
-// to h is computed exactly (Knuth's two-sum), that of the addition of those
-// errors to m likewise, and what is left goes to l.  72 bits against the 53 of
-// an FP64 accumulator, from FP32 additions only: this part issues two FP64
-// lanes per SM and clock, so that an FP64 add and conversion per cell took 32
-// of its clocks per warp against 3, and each of the ten dependent FP64 adds of
-// a block reduction about 300 clocks of latency against 100.
+// A sum kept as three floats: the rounding error of each addition to h is
+// computed exactly (Knuth's two-sum), that of the addition of those errors to m
+// likewise, and what is left goes to l.  Wider than the 53 bits of an FP64
+// accumulator, from FP32 additions only: this part issues two FP64 lanes per SM
+// and clock, so that an FP64 add and conversion per cell took 32 of its clocks
+// per warp against 3, and each of the ten dependent FP64 adds of a block
+// reduction about 300 clocks of latency against 100.
+// Every rounding is written out: a term that the compiler fuses as a product
+// into one addition of the two-sum and not into the other leaves an error of
+// 2^-24 of the term (3e-11 of the sum of |terms| over 60000 cells).
 struct Sum3 {
     float h, m, l;
 };
 __device__ __forceinline__ float two_sum(float& a, float b) {   // a += b; the exact error
-    const float t = a + b, z = t - a, e = (a - (t - z)) + (b - z);
+    const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
     a = t;
     return e;
 }
 __device__ __forceinline__ void sum3_add(Sum3& s, float x) {
     const float e = two_sum(s.h, x);
-    s.l += two_sum(s.m, e);
+    s.l = __fadd_rn(s.l, two_sum(s.m, e));
+}
+// s += x y, the product exact (its rounding error is the fused remainder).
+__device__ __forceinline__ void sum3_add_product(Sum3& s, float x, float y) {
+    const float p = __fmul_rn(x, y), q = __fmaf_rn(x, y, -p);
+    const float e = two_sum(s.h, p), f = two_sum(s.m, e);
+    s.l = __fadd_rn(s.l, __fadd_rn(f, two_sum(s.m, q)));
 }
 __device__ __forceinline__ void sum3_merge(Sum3& s, const Sum3& o) {
     const float e = two_sum(s.h, o.h), f = two_sum(s.m, o.m);
-    s.l = (s.l + o.l) + (f + two_sum(s.m, e));
+    s.l = __fadd_rn(__fadd_rn(s.l, o.l), __fadd_rn(f, two_sum(s.m, e)));
 }
 __device__ __forceinline__ double sum3_value(const Sum3& s) { return (double)s.h + ((double)s.m + (double)s.l); }
 __device__ __forceinline__ Sum3 warp_sum3(Sum3 v) {
@@ -494,10 +504,10 @@ struct CellUpdate {
                 emax = fmaxf(emax, en);
             }
         }
-        // the coupling sums: each cell's product in FP32, added without loss
+        // the coupling sums: m . B_rms,q in FP32, its product with Ms exact
 #pragma unroll
         for (int q = 0; q < NM; q++)
-            if (on[q]) sum3_add(xacc[q], Ms * (mx.x * px_[q] + mx.y * py_[q] + mx.z * pz_[q]));
+            if (on[q]) sum3_add_product(xacc[q], Ms, mx.x * px_[q] + mx.y * py_[q] + mx.z * pz_[q]);
         if constexpr (REC) {
             if (Ms > 0.f) { sum3_add(macc[0], mrec.x); sum3_add(macc[1], mrec.y); sum3_add(macc[2], mrec.z); }
         }

@@ -8,8 +8,8 @@
  * (omega_c, kappa, g, x0, p0) and integrator state (time, step size,
  * accept/reject counters).  Every step runs on the GPU: the zero-padded FFT
  * demag convolution, exchange, anisotropy, Zeeman, the cavity field
- * B_rms * Gamma(t) from a lossless (72-bit) reduction of the coupling-weighted
- * magnetisation, the LLG torque and the RK4 / Dormand-Prince update with |m|
+ * B_rms * Gamma(t) from a reduction of the coupling-weighted magnetisation
+ * (FP32 terms, sums wider than FP64), the LLG torque and the RK4 / Dormand-Prince update with |m|
  * renormalisation.  Nothing of the step runs on the host.
  *
  * Conventions for every call:
@@ -237,7 +237,7 @@ int mmcq_get_dt_history(mmcq_t* h, int inst, double* out, int64_t max, int64_t* 
  *   of mmcq_eval_field.
  * mmcq_set_recording: every > 0 records (t, <mx>, <my>, <mz>) of every
  *   instance after every `every`-th accepted step, <m> the mean of m over the
- *   magnetised cells (72-bit sums); 0 stops.  Capacity 65536 samples per
+ *   magnetised cells (sums of three floats, wider than FP64); 0 stops.  Capacity 65536 samples per
  *   instance (then MMCQ_ERR_STATE from the read-out).  First use allocates
  *   32 bytes x 65536 per instance.
  * mmcq_get_mavg_history: copies up to max samples of one instance into out

@@ -614,9 +614,10 @@ __global__ void __launch_bounds__(512, (FIXED && PH == 1024) ? 2 : 1) k_col_spli
 // order, but two stages at a time in registers (16 points per thread, 128
 // threads per column), so that each direction goes through shared memory three
 // times instead of six; the first pass reads global memory (rows of padding are
-// zeros in registers) and the last writes it.  Bound by instruction issue and
-// shared memory (104 KB, one block of 24 warps per SM).  1000x600 film:
-// 176 us (k_col_gen) -> 64 us per field evaluation.
+// zeros in registers) and the last writes it.  Bound by latency and L1: one
+// block of 24 warps per SM (104 KB, 80 registers), 3.4 waves of them; L1 and
+// shared memory 70 % busy, issue 42 %, the longest stall the twiddles' loads.
+// 1000x600 film: 176 us (k_col_gen) -> 64 us per field evaluation.
 //
 // Passes 1 and 2 (stages Ns, 4 Ns with Ns = 1, 16): thread t takes rows
 // t + 128 m; v[r' + 4 r''] is input r'' of butterfly t + 128 r' of the first

@@ -353,7 +353,12 @@ int rows_per_block(int L, int nrows) {
 // of 32 rows took 9.1 us in the x forward and 19.8 us in the x inverse, as 32
 // blocks of one row 3.2 and 6.2 us.  Measured at 1, 2 and 4 blocks per SM: a
 // 300x120x5 strip 1.42, 1.33 and 1.55 ms per 3 attempts, 16 films of 100x75
-// 4.13, 3.85 and 3.86 ms per 20 steps.
+// 4.13, 3.85 and 3.86 ms per 20 steps.  The same line serves rows of 256 and
+// 512 cells, whose compile-time shape needs four rows: a step of 512x512x1 takes
+// 147 us with the rule's two rows and 169 with four, 512x100x8 256 (three) and
+// 267, 256x256x2 128 (two) and 129, 256x40x16 152 (three) and 151; from four
+// rows on the fixed shape is the faster one (256x64x16: 155 and, with three,
+// 166 us).
 int rows_within(int most, long long rows_total, int sms) {
     long long R = (rows_total + 2LL * sms - 1) / (2LL * sms);
     return R < 1 ? 1 : (R > most ? most : (int)R);

@@ -3,8 +3,8 @@
 // giving B_demag, then exchange + anisotropy + Zeeman (with the Appendix C
 // excitation) + cavity sum_k B_rms,k Gamma_k (Sec. 2.1 field terms, Eq. bcav),
 // the LLG torque (Eq. llg), the RK bookkeeping, and block partials of the
-// coupling sums X_k = V_c sum_i Ms_i m_i . B_rms,k,i (Eq. gammafinal): each
-// cell's FP32 product added in three floats (Sum3).  The partials are reduced in
+// coupling sums X_k = V_c sum_i Ms_i m_i . B_rms,k,i (Eq. gammafinal): m . B in
+// FP32, its product with Ms exact, added in three floats (Sum3).  The partials are reduced in
 // a fixed order, and the cavity amplitudes and the step-size controller
 // advanced in FP64, by the scalar block of the next x forward or, at the end
 // of an attempt or of a call, by the instance's last block to finish.

@@ -23,8 +23,8 @@ __host__ __device__ constexpr int xpass_line_threads(int L) {
 constexpr int XPASS_F3_PADS = 4;
 __host__ __device__ constexpr int xpass_fft_rows(int L) { return xpass_f3(L) ? L + 16 * XPASS_F3_PADS : L; }
 
-// Threads of an x-pass block: 3 R lines x N1 threads per line with R = 64 / N1
-// rows (fewer when the grid has fewer rows), so never more than 192.
+// Most threads of an x-pass block: the 3 R lines x N1 threads per line of its
+// R <= 64 / N1 rows (fewer rows on a grid that would leave the GPU idle).
 constexpr int XPASS_THREADS = 192;
 // Resident blocks asked of the compiler: 5 (64 registers) while a thread
 // holds 16 points of the x transform, 3 when it holds 32 (L = 512).
